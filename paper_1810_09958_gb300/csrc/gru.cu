@@ -105,8 +105,11 @@ __host__ __device__ constexpr int gx_values(int ks, int bp) {
     return 3 * (kGroup / ks * bp / kGateThreads) * (bp == kBatchPad ? ks : 1);
 }
 
+// The partial rows of other CTAs' units that a CTA stages in a round.
+__host__ __device__ constexpr int stage_bytes(int ks, int bp) { return bp < 128 ? recv_bytes(bp) / ks * (ks - 1) : 0; }
+
 // [pad | next layer's W slice (has_next)] | h tile | 2 x partial rows |
-// 2 x projection values of a step | staged partial rows of other CTAs' units |
+// 2 x projection values of a step | kGruStages x staged partial rows |
 // barriers.  The pad: W's product starts 32 rows
 // before each atom.
 __host__ __device__ inline GruLayout gru_layout(int ks, int ka, bool has_next, int bp = kBatchPad) {
@@ -116,7 +119,7 @@ __host__ __device__ inline GruLayout gru_layout(int ks, int ka, bool has_next, i
     L.off_recv = L.off_h + ka * atom_h_bytes(bp);
     L.off_gx = L.off_recv + 2 * recv_bytes(bp);
     L.off_stage = L.off_gx + 2 * gx_values(ks, bp) * kGateThreads * 4;
-    L.off_bars = L.off_stage + (bp < 128 ? recv_bytes(bp) / ks * (ks - 1) : 0);
+    L.off_bars = L.off_stage + kGruStages * stage_bytes(ks, bp);
     L.total = L.off_bars + 192 + 1024;
     return L;
 }
@@ -436,7 +439,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         const uint32_t push_dst =
             mapa_shared(smem_u32(recv + ((static_cast<int>(rank) * 3 + (gate < 3 ? gate : 0)) * UO + oui) * BP), owner);
         const uint32_t push_bar = mapa_shared(smem_u32(red_full), owner);
-        // Bulk form: the quarter's rows staged as [other owner][UO units][BP].
+        // Bulk form: the quarter's rows staged as [round parity][gate][other owner][UO units][BP].
         const int peer = static_cast<int>(owner) - (owner > rank ? 1 : 0);
         uint8_t *stage = smem + L.off_stage + (gate < 3 ? gate : 0) * (kGroup - UO) * BP * 4;
         uint8_t *stage_row = stage + (peer * UO + oui) * BP * 4;
@@ -449,8 +452,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         auto push = [&](uint32_t par) {
             if (KS > 1 && BP < 128 && bulk)
                 push_rows_bulk<BP>(tmem_d + (static_cast<uint32_t>(gate * 32) << 16), half, npiece, owner != rank,
-                                   stage_row, push_dst + par * recv_bytes(BP), oui, push_bar + par * 8u, 1 + gate, sends,
-                                   stage_part, part_dst + par * recv_bytes(BP), part_bar + par * 8u,
+                                   stage_row + par * stage_bytes(KS, BP), push_dst + par * recv_bytes(BP), oui,
+                                   push_bar + par * 8u, 1 + gate, sends, stage_part + par * stage_bytes(KS, BP),
+                                   part_dst + par * recv_bytes(BP), part_bar + par * 8u,
                                    static_cast<uint32_t>(UO * BP * 4));
             else
                 push_rows<BP>(tmem_d + (static_cast<uint32_t>(gate * 32) << 16), half, npiece,

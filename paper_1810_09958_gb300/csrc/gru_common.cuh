@@ -159,13 +159,23 @@ __host__ __device__ inline bool gru_push_bulk(int batch, int bp) { return bp < 1
 // round takes 0.05 us longer (128 steps of two layers, hidden 1024: 395 -> 402 us).
 inline bool gru_dependent(int rounds) { return rounds <= 24; }
 
+// Staging buffers of push_rows_bulk, which rounds take in turn.
+constexpr int kGruStages = 2;
+
 // The same rows through a staging copy: warps w and w + 4 of a lane quarter each
 // write half of the columns of the rows of other CTAs (`remote`) to `stage`,
 // laid out as the owners hold them, then lane o of the first sends owner o's
 // `bytes` contiguous bytes as one bulk copy.  Whole rows move (padding
 // included); this CTA's own rows take the direct stores, npiece pieces each.
-// The stage is free again a round later: by then every owner has its rows, or
-// this CTA could not have gathered the round's vectors.
+//
+// A copy's end is seen on its owner's barrier only, so it is the exchange that lets
+// a buffer be written again, in round k + 2 after round k.  A CTA that has gathered
+// round k + 2's vectors has them from clusters that are through round k + 1; the CTAs
+// of one such cluster have, between them, gathered round k + 1's vectors of every CTA;
+// and an owner publishes those only after its rows of round k have landed.  One
+// buffer would not do: for round k + 1's vectors the same argument gives the rows of
+// round k - 1 only.  The second one takes 9 KB at 32 padded rows and four splits, 18
+// KB at 64 and 21 KB in the two-layer kernel.
 template <int BP>
 __device__ __forceinline__ void push_rows_bulk(uint32_t acc, int half, int npiece, bool remote, uint8_t *stage_row,
                                                uint32_t dst, int unit, uint32_t bar, int bar_id, bool sends,

@@ -56,6 +56,8 @@ constexpr int kRowBytes = kBatchPad * 4; // a received partial row
 // Rows per unit and source that a CTA receives: r, z, n of layer a; r, z, the
 // candidate's input and recurrent terms of layer b.
 __host__ __device__ constexpr int wave_rows(int layer) { return layer == 0 ? 3 : 4; }
+// Rows of the other CTAs' units that a CTA stages in a round.
+__host__ __device__ constexpr int wave_stage_bytes(int layer) { return wave_rows(layer) * (kGroup - kUO) * kRowBytes; }
 __host__ __device__ constexpr int wave_recv_bytes(int layer) { return kKS * wave_rows(layer) * kUO * kRowBytes; }
 // TMEM columns: layer a's accumulator, layer b's two (by round parity), then
 // the weights, 32 columns per K atom: U_a, W_b, U_b.
@@ -91,8 +93,8 @@ struct WaveLayout {
 };
 
 // h_a tile | h_b tile | partial rows of a, of b (2 round parities each) |
-// layer a's projection of 2 steps | staged partial rows of other CTAs' units of
-// a, of b | barriers.
+// layer a's projection of 2 steps | staged partial rows of a, of b (kGruStages
+// buffers each) | barriers.
 __host__ __device__ inline WaveLayout wave_layout(int ka) {
     WaveLayout L;
     L.off_h[0] = 0;
@@ -101,8 +103,8 @@ __host__ __device__ inline WaveLayout wave_layout(int ka) {
     L.off_recv[1] = L.off_recv[0] + 2 * wave_recv_bytes(0);
     L.off_gx = L.off_recv[1] + 2 * wave_recv_bytes(1);
     L.off_stage[0] = L.off_gx + 2 * 3 * 32 * kGateWarps * 4;
-    L.off_stage[1] = L.off_stage[0] + wave_rows(0) * (kGroup - kUO) * kRowBytes;
-    L.off_bars = L.off_stage[1] + wave_rows(1) * (kGroup - kUO) * kRowBytes;
+    L.off_stage[1] = L.off_stage[0] + kGruStages * wave_stage_bytes(0);
+    L.off_bars = L.off_stage[1] + kGruStages * wave_stage_bytes(1);
     L.total = L.off_bars + 256 + 1024;
     return L;
 }
@@ -240,7 +242,7 @@ __global__ void __launch_bounds__(kThreads, 1) gru_wave_kernel(const WaveParams 
             smem_u32(recv) + static_cast<uint32_t>(((static_cast<int>(rank) * rows + (q < rows ? q : 0)) * kUO + oui) * kRowBytes),
             owner);
         const uint32_t push_bar = mapa_shared(smem_u32(red), owner);
-        // Bulk form: the quarter's rows staged as [other owner][8 units][32].
+        // Bulk form: the quarter's rows staged as [round parity][row kind][other owner][8 units][32].
         const int qr = q < rows ? q : 0;
         const int peer = static_cast<int>(owner) - (owner > rank ? 1 : 0);
         uint8_t *stage = smem + L.off_stage[layer] + qr * (kGroup - kUO) * kRowBytes;
@@ -280,10 +282,12 @@ __global__ void __launch_bounds__(kThreads, 1) gru_wave_kernel(const WaveParams 
                 tc_fence_after();
                 const uint32_t acc_now = acc + (layer == 0 ? 0u : 32u * par);
                 const uint32_t buf = par * static_cast<uint32_t>(recv_buf);
+                const uint32_t stage_buf = par * static_cast<uint32_t>(wave_stage_bytes(layer));
                 if (p.bulk)
-                    push_rows_bulk<kBatchPad>(acc_now, half, npiece, owner != rank, stage_row, push_dst + buf, oui,
-                                              push_bar + par * 8u, 1 + 4 * layer + q, sends, stage_part, part_dst + buf,
-                                              part_bar + par * 8u, static_cast<uint32_t>(kUO * kRowBytes));
+                    push_rows_bulk<kBatchPad>(acc_now, half, npiece, owner != rank, stage_row + stage_buf, push_dst + buf,
+                                              oui, push_bar + par * 8u, 1 + 4 * layer + q, sends, stage_part + stage_buf,
+                                              part_dst + buf, part_bar + par * 8u,
+                                              static_cast<uint32_t>(kUO * kRowBytes));
                 else
                     push_rows<kBatchPad>(acc_now, half, npiece, push_dst + buf, oui, push_bar + par * 8u);
             }
