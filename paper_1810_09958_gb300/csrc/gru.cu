@@ -211,7 +211,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const GruLayout L = gru_layout(KS, p.ka, HN, BP);
     uint8_t *sW = smem + L.off_w;
     uint8_t *sH = smem + L.off_h;
-    float *recv = reinterpret_cast<float *>(smem + L.off_recv);  // [2 round parity][ks src][3 gates][uo][BP batch]
+    float *recv = reinterpret_cast<float *>(smem + L.off_recv);  // [2 round parity][ks src][3 gates][2 halves][uo][BP / 2]
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + L.off_bars);
     uint64_t *wbar = bars;                   // next layer's W slice landed
     uint64_t *h_full = bars + 1;             // the round's vectors are in shared memory
@@ -429,33 +429,30 @@ __global__ void __launch_bounds__(kThreads, 1)
         // the cluster CTA that owns unit u, into its slot for this source rank.
         // Warps w and w + 4 share the TMEM lane quarter w % 4 = the gate, each
         // taking half of the batch columns.  Round 0 of a reset-before step sends
-        // the r and z rows, round 1 the n rows.  16-byte piece c of a row sits at
-        // c ^ (row % 8), so that the gates' reads (8 or more rows, few batch
-        // columns per warp) fall into different banks.
+        // the r and z rows, round 1 the n rows.
         const int gate = warp & 3;
         const int half = warp >> 2;
         const uint32_t owner = static_cast<uint32_t>(lane / UO);
         const int oui = lane % UO;
-        const uint32_t push_dst =
-            mapa_shared(smem_u32(recv + ((static_cast<int>(rank) * 3 + (gate < 3 ? gate : 0)) * UO + oui) * BP), owner);
+        const int kind = ((static_cast<int>(rank) * 3 + (gate < 3 ? gate : 0)) * 2 + half) * UO;  // first half row at the owner
+        const uint32_t push_dst = mapa_shared(smem_u32(recv + (kind + oui) * (BP / 2)), owner);
         const uint32_t push_bar = mapa_shared(smem_u32(red_full), owner);
-        // Bulk form: the quarter's rows staged as [round parity][gate][other owner][UO units][BP].
+        // Bulk form: staged as [round parity][gate][half][other owner][UO units][BP / 2].
         const int peer = static_cast<int>(owner) - (owner > rank ? 1 : 0);
-        uint8_t *stage = smem + L.off_stage + (gate < 3 ? gate : 0) * (kGroup - UO) * BP * 4;
-        uint8_t *stage_row = stage + (peer * UO + oui) * BP * 4;
+        uint8_t *stage = smem + L.off_stage + ((gate < 3 ? gate : 0) * 2 + half) * (kGroup - UO) * (BP * 2);
+        uint8_t *stage_row = stage + (peer * UO + oui) * (BP * 2);
         const uint32_t to = static_cast<uint32_t>(lane & (KS - 1));  // lanes 0 .. KS - 1 send to owner `lane`
-        const bool sends = half == 0 && lane < KS && to != rank;
-        const uint32_t stage_part = smem_u32(stage) + (to - (to > rank ? 1u : 0u)) * static_cast<uint32_t>(UO * BP * 4);
-        const uint32_t part_dst =
-            mapa_shared(smem_u32(recv + (static_cast<int>(rank) * 3 + (gate < 3 ? gate : 0)) * UO * BP), to);
+        const bool sends = lane < KS && to != rank;
+        const uint32_t stage_part = smem_u32(stage) + (to - (to > rank ? 1u : 0u)) * static_cast<uint32_t>(UO * BP * 2);
+        const uint32_t part_dst = mapa_shared(smem_u32(recv + kind * (BP / 2)), to);
         const uint32_t part_bar = mapa_shared(smem_u32(red_full), to);
         auto push = [&](uint32_t par) {
             if (KS > 1 && BP < 128 && bulk)
                 push_rows_bulk<BP>(tmem_d + (static_cast<uint32_t>(gate * 32) << 16), half, npiece, owner != rank,
                                    stage_row + par * stage_bytes(KS, BP), push_dst + par * recv_bytes(BP), oui,
-                                   push_bar + par * 8u, 1 + gate, sends, stage_part + par * stage_bytes(KS, BP),
+                                   push_bar + par * 8u, sends, stage_part + par * stage_bytes(KS, BP),
                                    part_dst + par * recv_bytes(BP), part_bar + par * 8u,
-                                   static_cast<uint32_t>(UO * BP * 4));
+                                   static_cast<uint32_t>(UO * BP * 2));
             else
                 push_rows<BP>(tmem_d + (static_cast<uint32_t>(gate * 32) << 16), half, npiece,
                               push_dst + par * recv_bytes(BP), oui, push_bar + par * 8u);
@@ -538,7 +535,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 float ghr = bh_r, ghz = bh_z, ghn = bh_n;
 #pragma unroll
                 for (int s = 0; s < KS; ++s) {  // partials summed in rank order
-                    const float *rs = rv + (s * 3 * UO + ui) * BP + (((b >> 2) ^ (ui & 7)) << 2) + (b & 3);
+                    const float *rs = rv + s * 3 * UO * BP + recv_at<BP, UO>(ui, b);
                     if (!RB || ph == 0) {
                         ghr += rs[0];
                         ghz += rs[UO * BP];

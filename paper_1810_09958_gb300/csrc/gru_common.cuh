@@ -115,11 +115,27 @@ __device__ __forceinline__ bool gather_tile(const uint16_t *src, uint8_t *dst, u
     return true;
 }
 
+// Received partial rows: [source][row kind][half of the batch columns][unit][BP / 2],
+// each half written by another warp.  16-byte piece c of a unit's half sits at
+// c ^ recv_swizzle(unit), so that the gates' reads (8 or more units, few batch
+// columns per warp) fall into different banks.
+template <int BP>
+__device__ __forceinline__ int recv_swizzle(int unit) {
+    return BP == 32 ? (unit >> 1) & 3 : unit & 7;
+}
+
+// Floats from a row kind's first half to batch column b of a unit.
+template <int BP, int UO>
+__device__ __forceinline__ int recv_at(int unit, int b) {
+    const int half = b / (BP / 2), c = b % (BP / 2);
+    return (half * UO + unit) * (BP / 2) + (((c >> 2) ^ recv_swizzle<BP>(unit)) << 2) + (c & 3);
+}
+
 // Sends half `half` of the batch columns of this warp's 32 accumulator rows (at
-// `acc`, TMEM lane = row) to their owners: 16-byte piece c of a row goes to
-// piece c ^ (unit % 8) of the row at dst, counted on the owner's barrier `bar`;
-// only the npiece pieces that hold the batch are sent.  Asynchronous remote
-// stores: nothing here waits for them to land.
+// `acc`, TMEM lane = row) to their owners: dst is the half row in the owner's
+// received rows, counted on the owner's barrier `bar`; only the npiece pieces of
+// the whole row that hold the batch are sent.  Asynchronous remote stores: nothing
+// here waits for them to land.
 template <int BP>
 __device__ __forceinline__ void push_rows(uint32_t acc, int half, int npiece, uint32_t dst, int unit, uint32_t bar) {
     constexpr int CH = BP / 2 < 32 ? BP / 2 : 32;  // columns per TMEM load
@@ -136,7 +152,7 @@ __device__ __forceinline__ void push_rows(uint32_t acc, int half, int npiece, ui
 #pragma unroll
         for (int c = 0; c < CH / 4; ++c)
             if (col / 4 + c < npiece)
-                st_async_f4(dst + static_cast<uint32_t>(((col / 4 + c) ^ (unit & 7)) << 4),
+                st_async_f4(dst + static_cast<uint32_t>(((c0 / 4 + c) ^ recv_swizzle<BP>(unit)) << 4),
                             make_float4(__uint_as_float(r[4 * c]), __uint_as_float(r[4 * c + 1]),
                                         __uint_as_float(r[4 * c + 2]), __uint_as_float(r[4 * c + 3])),
                             bar);
@@ -162,11 +178,12 @@ inline bool gru_dependent(int rounds) { return rounds <= 24; }
 // Staging buffers of push_rows_bulk, which rounds take in turn.
 constexpr int kGruStages = 2;
 
-// The same rows through a staging copy: warps w and w + 4 of a lane quarter each
-// write half of the columns of the rows of other CTAs (`remote`) to `stage`,
-// laid out as the owners hold them, then lane o of the first sends owner o's
-// `bytes` contiguous bytes as one bulk copy.  Whole rows move (padding
-// included); this CTA's own rows take the direct stores, npiece pieces each.
+// The same half rows through a staging copy: the warp writes those of other CTAs
+// (`remote`) to `stage`, laid out as the owners hold them, then lane o sends owner
+// o's `bytes` contiguous bytes as one bulk copy.  Whole half rows move (padding
+// included); this CTA's own rows take the direct stores, npiece pieces each.  Warps
+// w and w + 4, which share a lane quarter, each send what they wrote: one that has
+// given up leaves the round, so no barrier may join them.
 //
 // A copy's end is seen on its owner's barrier only, so it is the exchange that lets
 // a buffer be written again, in round k + 2 after round k.  A CTA that has gathered
@@ -178,9 +195,8 @@ constexpr int kGruStages = 2;
 // KB at 64 and 21 KB in the two-layer kernel.
 template <int BP>
 __device__ __forceinline__ void push_rows_bulk(uint32_t acc, int half, int npiece, bool remote, uint8_t *stage_row,
-                                               uint32_t dst, int unit, uint32_t bar, int bar_id, bool sends,
-                                               uint32_t stage_part, uint32_t part_dst, uint32_t part_bar,
-                                               uint32_t bytes) {
+                                               uint32_t dst, int unit, uint32_t bar, bool sends, uint32_t stage_part,
+                                               uint32_t part_dst, uint32_t part_bar, uint32_t bytes) {
     constexpr int CH = BP / 2 < 32 ? BP / 2 : 32;
 #pragma unroll
     for (int c0 = 0; c0 < BP / 2; c0 += CH) {
@@ -193,7 +209,7 @@ __device__ __forceinline__ void push_rows_bulk(uint32_t acc, int half, int npiec
         tmem_ld_wait();
 #pragma unroll
         for (int c = 0; c < CH / 4; ++c) {
-            const uint32_t off = static_cast<uint32_t>(((col / 4 + c) ^ (unit & 7)) << 4);
+            const uint32_t off = static_cast<uint32_t>(((c0 / 4 + c) ^ recv_swizzle<BP>(unit)) << 4);
             if (remote)
                 *reinterpret_cast<uint4 *>(stage_row + off) = make_uint4(r[4 * c], r[4 * c + 1], r[4 * c + 2], r[4 * c + 3]);
             else if (col / 4 + c < npiece)
@@ -205,7 +221,7 @@ __device__ __forceinline__ void push_rows_bulk(uint32_t acc, int half, int npiec
     }
     tc_fence_before();
     fence_proxy_async_smem();
-    named_bar(static_cast<uint32_t>(bar_id), 64);
+    __syncwarp();
     if (sends) bulk_copy_cluster(part_dst, stage_part, bytes, part_bar);
     __syncwarp();
 }

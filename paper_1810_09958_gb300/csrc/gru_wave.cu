@@ -192,7 +192,7 @@ __global__ void __launch_bounds__(kThreads, 1) gru_wave_kernel(const WaveParams 
         uint8_t *sH = smem + L.off_h[layer];
         const int rows = wave_rows(layer);
         const int recv_buf = wave_recv_bytes(layer);
-        float *recv = reinterpret_cast<float *>(smem + L.off_recv[layer]);  // [2][src][row kind][unit][32]
+        float *recv = reinterpret_cast<float *>(smem + L.off_recv[layer]);  // [2][src][row kind][2 halves][unit][16]
         uint64_t *red = red_full + 2 * layer;
         // This CTA evaluates the gates of units unit0 + rank*8 + [0, 8); thread
         // ltid takes unit ltid % 8 and batch row ltid / 8.
@@ -238,20 +238,18 @@ __global__ void __launch_bounds__(kThreads, 1) gru_wave_kernel(const WaveParams 
         const bool pushes = q < rows && (p.bulk || half * (kBatchPad / 8) < npiece);
         const uint32_t owner = static_cast<uint32_t>(lane / kUO);
         const int oui = lane % kUO;
-        const uint32_t push_dst = mapa_shared(
-            smem_u32(recv) + static_cast<uint32_t>(((static_cast<int>(rank) * rows + (q < rows ? q : 0)) * kUO + oui) * kRowBytes),
-            owner);
-        const uint32_t push_bar = mapa_shared(smem_u32(red), owner);
-        // Bulk form: the quarter's rows staged as [round parity][row kind][other owner][8 units][32].
         const int qr = q < rows ? q : 0;
+        const int kind = ((static_cast<int>(rank) * rows + qr) * 2 + half) * kUO;  // first half row at the owner
+        const uint32_t push_dst = mapa_shared(smem_u32(recv) + static_cast<uint32_t>((kind + oui) * (kRowBytes / 2)), owner);
+        const uint32_t push_bar = mapa_shared(smem_u32(red), owner);
+        // Bulk form: staged as [round parity][row kind][half][other owner][8 units][16].
         const int peer = static_cast<int>(owner) - (owner > rank ? 1 : 0);
-        uint8_t *stage = smem + L.off_stage[layer] + qr * (kGroup - kUO) * kRowBytes;
-        uint8_t *stage_row = stage + (peer * kUO + oui) * kRowBytes;
+        uint8_t *stage = smem + L.off_stage[layer] + (qr * 2 + half) * (kGroup - kUO) * (kRowBytes / 2);
+        uint8_t *stage_row = stage + (peer * kUO + oui) * (kRowBytes / 2);
         const uint32_t to = static_cast<uint32_t>(lane % kKS);  // lanes 0 .. 3 send to owner `lane`
-        const bool sends = half == 0 && lane < kKS && to != rank;
-        const uint32_t stage_part = smem_u32(stage) + (to - (to > rank ? 1u : 0u)) * static_cast<uint32_t>(kUO * kRowBytes);
-        const uint32_t part_dst = mapa_shared(
-            smem_u32(recv) + static_cast<uint32_t>((static_cast<int>(rank) * rows + qr) * kUO * kRowBytes), to);
+        const bool sends = lane < kKS && to != rank;
+        const uint32_t stage_part = smem_u32(stage) + (to - (to > rank ? 1u : 0u)) * static_cast<uint32_t>(kUO * kRowBytes / 2);
+        const uint32_t part_dst = mapa_shared(smem_u32(recv) + static_cast<uint32_t>(kind * (kRowBytes / 2)), to);
         const uint32_t part_bar = mapa_shared(smem_u32(red), to);
         const uint32_t acc = tmem + (static_cast<uint32_t>(q * 32) << 16) + (layer == 0 ? kColA : kColB);
 
@@ -285,9 +283,8 @@ __global__ void __launch_bounds__(kThreads, 1) gru_wave_kernel(const WaveParams 
                 const uint32_t stage_buf = par * static_cast<uint32_t>(wave_stage_bytes(layer));
                 if (p.bulk)
                     push_rows_bulk<kBatchPad>(acc_now, half, npiece, owner != rank, stage_row + stage_buf, push_dst + buf,
-                                              oui, push_bar + par * 8u, 1 + 4 * layer + q, sends, stage_part + stage_buf,
-                                              part_dst + buf, part_bar + par * 8u,
-                                              static_cast<uint32_t>(kUO * kRowBytes));
+                                              oui, push_bar + par * 8u, sends, stage_part + stage_buf, part_dst + buf,
+                                              part_bar + par * 8u, static_cast<uint32_t>(kUO * kRowBytes / 2));
                 else
                     push_rows<kBatchPad>(acc_now, half, npiece, push_dst + buf, oui, push_bar + par * 8u);
             }
@@ -304,7 +301,7 @@ __global__ void __launch_bounds__(kThreads, 1) gru_wave_kernel(const WaveParams 
                 break;
             }
             // Partials summed over the 4 source ranks in rank order.
-            const float *rv = recv + par * (recv_buf / 4) + ui * kBatchPad + (((b >> 2) ^ ui) << 2) + (b & 3);
+            const float *rv = recv + par * (recv_buf / 4) + recv_at<kBatchPad, kUO>(ui, b);
             auto part = [&](int src, int kind) { return rv[(src * rows + kind) * kUO * kBatchPad]; };
             float gr = bh_r, gz = bh_z, gn = bh_n;
 #pragma unroll

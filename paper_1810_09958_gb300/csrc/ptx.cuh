@@ -527,8 +527,9 @@ __device__ __forceinline__ void bulk_copy_cluster(uint32_t dst, uint32_t src, ui
         : "memory");
 }
 
-// Named barrier over `count` threads that also ANDs a predicate across them:
-// every participant gets the same result.
+// Named barrier over `count` threads (ids 1..15; 0 is __syncthreads) that also
+// ANDs a predicate across them: every participant gets the same result.  It is
+// not bounded, so every participant comes to it, also after a wait that ran out.
 __device__ __forceinline__ bool named_bar_and(uint32_t id, uint32_t count, bool pred) {
     uint32_t r;
     asm volatile(
@@ -540,11 +541,6 @@ __device__ __forceinline__ bool named_bar_and(uint32_t id, uint32_t count, bool 
         : "r"(pred ? 1u : 0u), "r"(id), "r"(count)
         : "memory");
     return r != 0;
-}
-
-// Named barrier over `count` threads (ids 1..15; 0 is __syncthreads).
-__device__ __forceinline__ void named_bar(uint32_t id, uint32_t count) {
-    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
 }
 
 }  // namespace isam

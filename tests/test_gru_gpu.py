@@ -115,10 +115,12 @@ def test_gru_unsupported_shapes_rejected():
 
 
 @pytest.mark.parametrize("reset_before", [False, True])
-def test_gru_missing_participant_times_out_cleanly(reset_before):
-    """One CTA never signals the step counter (a flag nothing sets): every
-    bounded wait runs out, the kernel returns, isam_sync reports
-    ISAM_ERR_TIMEOUT, and the context stays usable for a correct call."""
+@pytest.mark.parametrize("batch,H", [(8, 128), (32, 128), (64, 256)])
+def test_gru_missing_participant_times_out_cleanly(reset_before, batch, H):
+    """One CTA never publishes its states (words nothing sets): every bounded
+    wait runs out, the kernel returns, isam_sync reports ISAM_ERR_TIMEOUT, and
+    the context stays usable for a correct call.  The partial rows cross the
+    cluster as single stores at batch 8 and as bulk copies at 32 and 64."""
     rb = bool(reset_before)
     code = textwrap.dedent(f"""
         import sys, numpy as np, torch
@@ -128,7 +130,7 @@ def test_gru_missing_participant_times_out_cleanly(reset_before):
         import oracle
         from gpu_util import dev_bf16, nmax_err
         torch.cuda.set_device(0)
-        T, batch, H = 4, 8, 128
+        T, batch, H = 4, {batch}, {H}
         x, W, U, b, h0 = synth.gru_operands(T, batch, H, seed=3)
         args = [dev_bf16(x), dev_bf16(W), dev_bf16(U), torch.from_numpy(b).cuda(), None]
         out = torch.zeros(T * batch * H, device="cuda")

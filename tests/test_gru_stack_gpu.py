@@ -150,10 +150,12 @@ def test_gru_stack_pairs_and_per_layer_chain_agree(L, monkeypatch):
     assert np.array_equal(pairs[0], chain[0])
 
 
-def test_gru_stack_pair_kernel_missing_participant_times_out_cleanly():
-    """One CTA of the two-layer kernel never signals the round counter (a flag
-    nothing sets): every bounded wait runs out, the kernel returns, isam_sync
-    reports ISAM_ERR_TIMEOUT, and a correct call works afterwards."""
+@pytest.mark.parametrize("batch", [8, 32])
+def test_gru_stack_pair_kernel_missing_participant_times_out_cleanly(batch):
+    """One CTA of the two-layer kernel never publishes its states (words nothing
+    sets): every bounded wait runs out, the kernel returns, isam_sync reports
+    ISAM_ERR_TIMEOUT, and a correct call works afterwards.  The partial rows
+    cross the cluster as single stores at batch 8, as bulk copies at 32."""
     import os
     import subprocess
     import sys
@@ -166,7 +168,7 @@ def test_gru_stack_pair_kernel_missing_participant_times_out_cleanly():
         import oracle
         from gpu_util import dev_bf16, nmax_err
         torch.cuda.set_device(0)
-        L, T, batch, H = 2, 4, 8, 256
+        L, T, batch, H = 2, 4, {batch}, 256
         x, W, U, b, h0 = synth.gru_stack_operands(L, T, batch, H, seed=97)
         args = [dev_bf16(x), dev_bf16(W), dev_bf16(U), torch.from_numpy(b.reshape(-1)).cuda(), None]
         out = torch.zeros(L * T * batch * H, device="cuda")

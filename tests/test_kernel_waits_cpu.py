@@ -1,0 +1,19 @@
+"""Every wait of a kernel is bounded: what the sources may hold, checked as text."""
+import glob
+import os
+import re
+
+from paper_1810_09958_gb300 import build
+
+
+def kernel_sources():
+    for path in sorted(glob.glob(os.path.join(build.CSRC, "*.cu*"))):
+        with open(path) as f:
+            yield os.path.basename(path), re.sub(r"//[^\n]*", "", f.read())
+
+
+def test_no_barrier_joins_warps_that_may_have_given_up():
+    """A warp whose bounded wait ran out leaves its loop, so a plain named
+    barrier could hold the warps that wait for it for ever."""
+    for name, text in kernel_sources():
+        assert "bar.sync" not in text and "barrier.sync" not in text, name
