@@ -17,3 +17,11 @@ def test_no_barrier_joins_warps_that_may_have_given_up():
     barrier could hold the warps that wait for it for ever."""
     for name, text in kernel_sources():
         assert "bar.sync" not in text and "barrier.sync" not in text, name
+
+
+def test_only_the_depthwise_loop_keeps_a_named_barrier():
+    """Its warps come to it whatever their waits said, and leave together.  In the
+    GEMM's split epilogue a warp could leave at the accumulator's wait while the
+    others went on to the barrier."""
+    users = [name for name, text in kernel_sources() if re.search(r"\bnamed_bar_and\(", text) and name != "ptx.cuh"]
+    assert users == ["depthwise.cu"], users
