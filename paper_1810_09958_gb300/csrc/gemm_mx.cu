@@ -429,18 +429,8 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_mx_kernel(const __grid_const
                 }
                 if (!load_c && lead) bulk_wait_read<1>();
                 uint32_t r[32];
-                if (pr.bn - j * 32 >= 32) {
-                    tmem_ld32(tbase + j * 32, r);
-                } else {
-                    uint32_t h[16];
-                    tmem_ld16(tbase + j * 32, h);
-#pragma unroll
-                    for (int i = 0; i < 16; ++i) {
-                        r[i] = h[i];
-                        r[16 + i] = 0u;
-                    }
-                }
-                tmem_ld_wait();
+                tmem_ld32(tbase + j * 32, r);  // past bn: columns of the accumulator's own 128, never stored
+                tmem_ld_wait(r);
                 if (load_c) {
                     if (!warp_wait(&cb[b], cpar[b], w, SITE_X_CLOAD)) {
                         ok = false;

@@ -148,7 +148,7 @@ __device__ __forceinline__ void push_rows(uint32_t acc, int half, int npiece, ui
             tmem_ld16(acc + static_cast<uint32_t>(col), r);
         else
             tmem_ld32(acc + static_cast<uint32_t>(col), r);
-        tmem_ld_wait();
+        tmem_ld_wait(r);
 #pragma unroll
         for (int c = 0; c < CH / 4; ++c)
             if (col / 4 + c < npiece)
@@ -206,7 +206,7 @@ __device__ __forceinline__ void push_rows_bulk(uint32_t acc, int half, int npiec
             tmem_ld16(acc + static_cast<uint32_t>(col), r);
         else
             tmem_ld32(acc + static_cast<uint32_t>(col), r);
-        tmem_ld_wait();
+        tmem_ld_wait(r);
 #pragma unroll
         for (int c = 0; c < CH / 4; ++c) {
             const uint32_t off = static_cast<uint32_t>(((c0 / 4 + c) ^ recv_swizzle<BP>(unit)) << 4);

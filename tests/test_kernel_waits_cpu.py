@@ -25,3 +25,12 @@ def test_only_the_depthwise_loop_keeps_a_named_barrier():
     others went on to the barrier."""
     users = [name for name, text in kernel_sources() if re.search(r"\bnamed_bar_and\(", text) and name != "ptx.cuh"]
     assert users == ["depthwise.cu"], users
+
+
+def test_every_wait_for_a_tensor_memory_load_names_its_registers():
+    """The load fills its registers asynchronously: work on them could otherwise
+    be moved ahead of the wait."""
+    for name, text in kernel_sources():
+        assert "tmem_ld_wait()" not in text, name
+        for asm in re.findall(r'"tcgen05\.wait::ld[^;]*;"\s*:(.)', text):
+            assert asm != ":", name
