@@ -58,14 +58,14 @@ constexpr uint32_t kTmemCols = 512;        // 2 accumulators x 128 + scale ring
 constexpr uint32_t kSfCol0 = 2 * kBNMax;   // first column of the scale ring
 
 enum : uint32_t {
-    SITE_X_EMPTY = 0x501,
-    SITE_X_TEMPTY = 0x502,
-    SITE_X_FULL = 0x503,
-    SITE_X_SFULL = 0x504,
-    SITE_X_TFULL = 0x505,
-    SITE_X_CLOAD = 0x506,
-    SITE_X_SEMPTY = 0x507,
-    SITE_X_DONE = 0x508,
+    SITE_X_EMPTY = 0x701,
+    SITE_X_TEMPTY = 0x702,
+    SITE_X_FULL = 0x703,
+    SITE_X_SFULL = 0x704,
+    SITE_X_TFULL = 0x705,
+    SITE_X_CLOAD = 0x706,
+    SITE_X_SEMPTY = 0x707,
+    SITE_X_DONE = 0x708,
 };
 
 struct MxProblem {
@@ -136,7 +136,7 @@ __host__ __device__ inline int mx_epi_bytes(int bn, int log_split) { return log_
 template <int CAP>
 __global__ void __launch_bounds__(kThreads, 1) gemm_mx_kernel(const __grid_constant__ MxParams<CAP> p) {
     const int ls = CAP == 1 ? p.log_split : 0;
-    if (ls > 0 && !launch_shape_ok(p.err, 1u << ls, gridDim.x, 0x5F0u)) return;
+    if (ls > 0 && !launch_shape_ok(p.err, 1u << ls, gridDim.x, 0x7F0u)) return;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                                 ~static_cast<uintptr_t>(1023));

@@ -34,3 +34,11 @@ def test_every_wait_for_a_tensor_memory_load_names_its_registers():
         assert "tmem_ld_wait()" not in text, name
         for asm in re.findall(r'"tcgen05\.wait::ld[^;]*;"\s*:(.)', text):
             assert asm != ":", name
+
+
+def test_error_sites_belong_to_one_kernel_each():
+    """isam_sync reports the site and block alone."""
+    sites = [(code, name) for name, text in kernel_sources()
+             for code in re.findall(r"\bSITE_\w+ = (0x[0-9A-Fa-f]+)", text) + re.findall(r"\b(0x[0-9A-Fa-f]{3})u\)", text)]
+    codes = [int(code, 16) for code, _ in sites]
+    assert len(codes) > 40 and len(set(codes)) == len(codes), sorted(sites)
