@@ -78,6 +78,38 @@ __device__ __forceinline__ void split_push(uint8_t *stage, const void *recv, con
     }
 }
 
+// The same without staging the tile: the warp turns a chunk of its 32 rows around
+// in `buf` (4 KB) and stores it into the owners' `recv`, each instruction whole rows
+// of the chunk, 16 bytes a thread.
+template <typename Load>
+__device__ __forceinline__ void split_store(uint8_t *buf, const void *recv, const uint64_t *full, int q, int lane,
+                                            uint32_t rank, int ls, int cw, int nch, Load load, int first, int step) {
+    const int lr = 7 - ls, rowb = cw * 4, lp = cw == 32 ? 3 : 2;
+    const uint32_t slot = smem_u32(recv) + static_cast<uint32_t>((static_cast<int>(rank) * nch << lr) * rowb);
+    const uint32_t bar = smem_u32(full);
+#pragma unroll 1
+    for (int c = first; c < nch; c += step) {
+        uint32_t r[32];
+        load(c * cw, r);
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+            if (j < 4 || cw == 32)
+                *reinterpret_cast<uint4 *>(buf + lane * rowb + ((j ^ split_swizzle(cw, lane)) << 4)) =
+                    make_uint4(r[4 * j], r[4 * j + 1], r[4 * j + 2], r[4 * j + 3]);
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            if (i >= 4 && cw != 32) break;
+            const int at = i * 32 + lane, row = q * 32 + (at >> lp);  // the piece stays where the swizzle put it
+            const float4 v = *reinterpret_cast<const float4 *>(buf + at * 16);
+            const uint32_t owner = static_cast<uint32_t>(row >> lr);
+            const uint32_t off = static_cast<uint32_t>(((c << lr) + (row & ((1 << lr) - 1))) * rowb + ((at & ((1 << lp) - 1)) << 4));
+            st_async_f4(mapa_shared(slot + off, owner), v, mapa_shared(bar, owner));
+        }
+        __syncwarp();
+    }
+}
+
 // Sums the slices this CTA received, in rank order, by `threads` threads (t), and
 // stores alpha * sum + bias + beta * C: rows r0 on, `width` columns from col0 on.
 __device__ __forceinline__ void split_sum(const void *recv, int t, int threads, int ls, int cw, int nch, int r0,

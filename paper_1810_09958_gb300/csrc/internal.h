@@ -112,6 +112,9 @@ struct GemmPlan {
     size_t smem;  // dynamic shared memory bytes
     double est_us;
     int pair = 0; // 1: 256 x 256 tiles on CTA pairs (cta_group::2), see gemm_pair.cu
+    int parts = 1;  // accumulators a tile's K range is spread over
+    int bufs = 2;   // 2: the next tile's accumulators fit beside this one's
+    int walk = 0;   // split tiles: a cluster has more than one
 };
 
 int gemm_validate(const GemmDesc &g);
