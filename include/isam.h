@@ -216,6 +216,16 @@ int isam_gemm_plan_for(int M, int N, int K, int transA, int transB, float beta, 
                        const int *cluster_caps, int *out);
 
 /*
+ * The longest running sum of that plan: out[0] = 64-wide K atoms that one
+ * fp32 accumulator of the tensor cores adds up (what the plan splits K into,
+ * over CTAs or accumulators, is added in fp32 afterwards).  The running sum
+ * loses about 6e-8 of the result per atom.  Arguments and errors as for
+ * isam_gemm_plan_for.
+ */
+int isam_gemm_chain_for(int M, int N, int K, int transA, int transB, float beta, int num_sms, int smem_optin,
+                        const int *cluster_caps, int *out);
+
+/*
  * GRU forward inference over T steps (input size == hidden).
  *
  * The recurrent model the paper schedules with a priming, a recursive and a

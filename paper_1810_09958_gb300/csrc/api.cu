@@ -475,10 +475,12 @@ int isam_gemm_plan_info2(int M, int N, int K, int transA, int transB, float beta
     return ISAM_OK;
 }
 
-int isam_gemm_plan_for(int M, int N, int K, int transA, int transB, float beta, int num_sms, int smem_optin,
-                       const int *cluster_caps, int *out) {
+namespace {
+// The plan of a GEMM for given limits; `who` names the call in errors.
+int plan_for(const char *who, int M, int N, int K, int transA, int transB, float beta, int num_sms, int smem_optin,
+             const int *cluster_caps, const int *out, GemmPlan *plan) {
     if (!out || !cluster_caps || num_sms < 1 || smem_optin < 1)
-        return set_error(ISAM_ERR_INVALID_ARG, "isam_gemm_plan_for: null output or limits < 1");
+        return set_error(ISAM_ERR_INVALID_ARG, "%s: null output or limits < 1", who);
     GemmDesc g{M, N, K, transA, transB, 1.0f, beta, reinterpret_cast<const uint16_t *>(16),
                reinterpret_cast<const uint16_t *>(16), reinterpret_cast<float *>(16), nullptr};
     int rc = gemm_validate(g);
@@ -487,12 +489,19 @@ int isam_gemm_plan_for(int M, int N, int K, int transA, int transB, float beta, 
     ds.num_sms = num_sms;
     ds.max_smem_optin = smem_optin;
     for (int i = 0; i < 3; ++i) {
-        if (cluster_caps[i] < 1)
-            return set_error(ISAM_ERR_INVALID_ARG, "isam_gemm_plan_for: cluster capacities must be >= 1");
+        if (cluster_caps[i] < 1) return set_error(ISAM_ERR_INVALID_ARG, "%s: cluster capacities must be >= 1", who);
         ds.cluster_cap[i] = cluster_caps[i];
     }
+    return gemm_plan(g, ds, plan);
+}
+}  // namespace
+
+int isam_gemm_plan_for(int M, int N, int K, int transA, int transB, float beta, int num_sms, int smem_optin,
+                       const int *cluster_caps, int *out) {
     GemmPlan plan;
-    if ((rc = gemm_plan(g, ds, &plan))) return rc;
+    if (const int rc = plan_for("isam_gemm_plan_for", M, N, K, transA, transB, beta, num_sms, smem_optin, cluster_caps,
+                                out, &plan))
+        return rc;
     out[0] = plan.BN;
     out[1] = plan.split;
     out[2] = plan.stages;
@@ -501,6 +510,16 @@ int isam_gemm_plan_for(int M, int N, int K, int transA, int transB, float beta, 
     out[5] = static_cast<int>(plan.smem);
     out[6] = plan.pair ? 256 : 128;
     out[7] = plan.pair ? 2 : 1;
+    return ISAM_OK;
+}
+
+int isam_gemm_chain_for(int M, int N, int K, int transA, int transB, float beta, int num_sms, int smem_optin,
+                        const int *cluster_caps, int *out) {
+    GemmPlan plan;
+    if (const int rc = plan_for("isam_gemm_chain_for", M, N, K, transA, transB, beta, num_sms, smem_optin,
+                                cluster_caps, out, &plan))
+        return rc;
+    out[0] = plan.chain;
     return ISAM_OK;
 }
 

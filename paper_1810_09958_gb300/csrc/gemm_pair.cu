@@ -402,6 +402,7 @@ int gemm_pair_plan(const GemmDesc &g, const DeviceState &ds, GemmPlan *plan) {
     p.grid = static_cast<int>(std::min<long long>(tiles, pairs)) * 2;
     p.smem = pair_smem_bytes(st);
     p.pair = 1;
+    p.chain = (g.K + kBK - 1) / kBK;
     p.est_us = 0.0;
     *plan = p;
     return 1;

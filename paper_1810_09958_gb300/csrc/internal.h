@@ -114,6 +114,7 @@ struct GemmPlan {
     int pair = 0; // 1: 256 x 256 tiles on CTA pairs (cta_group::2), see gemm_pair.cu
     int parts = 1;  // accumulators a tile's K range is spread over
     int bufs = 2;   // 2: the next tile's accumulators fit beside this one's
+    int chain = 0;  // K atoms of the longest running sum in one accumulator
     int walk = 0;   // split tiles: a cluster has more than one
 };
 

@@ -72,6 +72,7 @@ def load():
         lib.isam_dwsep_plan_info.argtypes = [i, i, i, P]
         lib.isam_dwsep_plan_for.argtypes = [i, i, i, i, P]
         lib.isam_gemm_plan_for.argtypes = [i, i, i, i, i, f, i, i, P, P]
+        lib.isam_gemm_chain_for.argtypes = [i, i, i, i, i, f, i, i, P, P]
         lib.isam_gru_plan_info.argtypes = [i, i, i, i, P]
         lib.isam_gru_plan_for.argtypes = [i, i, i, i, i, i, P]
         for name in ("isam_version", "isam_set_stream", "isam_sync", "isam_shutdown", "isam_gemm",
@@ -80,7 +81,7 @@ def load():
                      "isam_gru_forward", "isam_gru_forward_reset_before",
                      "isam_gru_forward_stack",
                      "isam_dwsep_conv", "isam_dwsep_plan_info", "isam_dwsep_plan_for", "isam_depthwise_conv3x3",
-                     "isam_gru_plan_info", "isam_gru_plan_for", "isam_gemm_plan_for"):
+                     "isam_gru_plan_info", "isam_gru_plan_for", "isam_gemm_plan_for", "isam_gemm_chain_for"):
             getattr(lib, name).restype = ctypes.c_int
         _lib = lib
         return lib
@@ -295,6 +296,15 @@ def gemm_plan(M, N, K, transA, transB, beta=0.0, num_sms=None, smem_optin=None, 
         caps = (ctypes.c_int * 3)(*cluster_caps)
         check(lib.isam_gemm_plan_for(M, N, K, int(transA), int(transB), float(beta), num_sms, smem_optin, caps, out))
     return dict(zip(("BN", "split", "stages", "group_m", "grid", "smem", "tile_m", "cta_pair"), list(out)))
+
+
+def gemm_chain(M, N, K, transA, transB, beta=0.0, *, num_sms, smem_optin, cluster_caps) -> int:
+    """isam_gemm_chain_for: 64-wide K atoms in the longest running sum of the plan."""
+    lib = load()
+    out = (ctypes.c_int * 1)()
+    caps = (ctypes.c_int * 3)(*cluster_caps)
+    check(lib.isam_gemm_chain_for(M, N, K, int(transA), int(transB), float(beta), num_sms, smem_optin, caps, out))
+    return out[0]
 
 
 def gru_forward(T, batch, hidden, x, W, U, b, h0, h_out, reset_before=False) -> None:

@@ -166,6 +166,24 @@ def test_gemm_output_chunks_of_two_warps(M, N, K, bn, beta, monkeypatch):
     assert np.array_equal(got.astype(np.float64), ref)
 
 
+@pytest.mark.parametrize("M,N,K,tA,tB,beta", [(520, 3880, 1800, 0, 0, 0.0), (528, 3848, 1832, 1, 1, 1.0)])
+def test_gemm_several_tiles_in_a_single_buffer(M, N, K, tA, tB, beta):
+    """A plan that spends all of TMEM on one tile's sums although CTAs have
+    several tiles (155 on 152 SMs, three accumulators of 128 columns).  Integer
+    data exact."""
+    import torch
+    plan = isam.gemm_plan(M, N, K, tA, tB, beta)
+    tiles = -(-M // 128) * -(-N // plan["BN"])
+    chain = isam.gemm_chain(M, N, K, tA, tB, beta, num_sms=torch.cuda.get_device_properties(0).multi_processor_count,
+                            smem_optin=232448, cluster_caps=[76, 36, 16])
+    assert (plan["BN"], plan["split"]) == (128, 1) and tiles > plan["grid"]
+    assert chain * 2 < -(-K // 64)  # more accumulators than fit twice
+    A, B, C0 = synth.gemm_operands(M, N, K, tA, tB, seed=600 + M, dist="int4", beta_c=True)
+    got = run_gemm(M, N, K, tA, tB, 2.0, beta, A, B, C0=C0)
+    ref = oracle.gemm(M, N, K, tA, tB, 2.0, A, B, beta, C0)
+    assert np.array_equal(got.astype(np.float64), ref)
+
+
 def test_gemm_split_k_deterministic(monkeypatch):
     monkeypatch.setenv("ISAM_FORCE_TILE", "64,8,0")
     M, N, K = 1760, 64, 1760

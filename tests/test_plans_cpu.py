@@ -186,6 +186,27 @@ def test_gemm_plans_over_a_grid_of_shapes():
                         check_gemm_plan(M, N, K, tA, tB, gemm_plan(M, N, K, tA, tB))
 
 
+# K atoms (64 elements) that K over the split of a streaming model leaves to a CTA,
+# for shapes whose fastest plan sums several times as many in one accumulator.
+CHAINS = [
+    ((3608, 750, 2376, 0, 1), 10), ((822, 1937, 4592, 0, 1), 9), ((2803, 864, 5280, 0, 1), 21),
+    ((1768, 1432, 4251, 1, 0), 17), ((848, 6392, 4817, 1, 0), 38), ((4392, 1191, 4560, 1, 1), 36),
+    ((8128, 531, 3840, 1, 1), 15), ((6440, 1481, 3480, 1, 1), 14), ((4392, 2248, 2642, 1, 0), 21),
+    ((4168, 1432, 4283, 1, 0), 17), ((3952, 2608, 5071, 1, 0), 40), ((2808, 1890, 4336, 0, 1), 34),
+    ((4065, 1438, 6576, 0, 1), 26), ((4872, 1192, 2437, 1, 0), 10), ((736, 8160, 2895, 1, 0), 12),
+    ((2136, 1032, 7387, 1, 0), 29),
+]
+
+
+@pytest.mark.parametrize("shape,atoms", CHAINS, ids=[str(s) for s, _ in CHAINS])
+def test_gemm_running_sums_stay_as_short_as_the_split_of_a_streaming_model(shape, atoms):
+    """The tensor cores' running sum loses about 6e-8 of the result per K atom; sums
+    of up to 14 atoms are not shortened further."""
+    caps = [76, 36, 16]  # clusters of 2, 4 and 8 CTAs that a GB300 holds
+    for beta in (0.0, 1.0):
+        assert isam.gemm_chain(*shape, beta, num_sms=SMS, smem_optin=SMEM, cluster_caps=caps) <= max(14, atoms)
+
+
 def test_gemm_plans_with_few_resident_clusters():
     for (M, N, K) in [(4096, 16, 4096), (8192, 8192, 8192), (512, 512, 512)]:
         check_gemm_plan(M, N, K, 0, 0, gemm_plan(M, N, K, 0, 0, caps=[1, 1, 1]))
