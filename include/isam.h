@@ -402,15 +402,38 @@ int isam_depthwise_conv3x3(int N, int H, int W, int C, const isam_bf16 *x, const
                            isam_bf16 *y);
 
 /*
- * A static tiling of a separable layer for images W pixels wide with Cin ->
- * Cout channels; nothing is launched.  It does not depend on N or H:
- * isam_dwsep_conv, which knows them, runs patches of 128 pixels (8 x 16, 16 x 8
- * or 4 x 32) and shares the output channels out over as few CTAs per patch as
- * its shared memory and the idle SMs call for.  out[4]:
- *   out[0]  0 = a 128-pixel tile can hold whole image rows with their input
- *           rows in shared memory, 1 = it cannot
- *   out[1]  image rows per tile (out[0] = 0), else 0
- *   out[2]  output-channel blocks whose weights fit beside such a tile
+ * How isam_dwsep_conv runs a layer; nothing is launched.  out[9]:
+ *   out[0]  columns of a patch of pixels (16, 8 or 32; a patch has 128 pixels of
+ *           one image)
+ *   out[1]  rows of a patch
+ *   out[2]  patches of all images
+ *   out[3]  output-channel blocks: as few as the shared memory allows, more
+ *           where SMs would be idle; each recomputes the depthwise stage
+ *   out[4]  channels per block: all of them, or a multiple of 32 (the last
+ *           block may have fewer)
+ *   out[5]  CTAs per block, which walk the patches
+ *   out[6]  64-channel chunks of patches in flight
+ *   out[7]  64-channel chunks of depthwise results in flight
+ *   out[8]  shared memory of a CTA in bytes
+ * ISAM_ERR_UNSUPPORTED for sizes isam_dwsep_conv rejects, ISAM_ERR_INVALID_ARG
+ * for sizes < 1 or a null out.
+ */
+int isam_dwsep_call_info(int N, int H, int W, int Cin, int Cout, int *out);
+
+/*
+ * The same for a device with num_sms SMs (152 on a GB300) whose CTAs may opt in
+ * to smem_optin bytes of shared memory (232448 on sm_103a); host arithmetic
+ * only, no CUDA call, so it runs without a GPU.
+ */
+int isam_dwsep_call_for(int N, int H, int W, int Cin, int Cout, int num_sms, int smem_optin, int *out);
+
+/*
+ * What of that plan the width and the channel counts fix, for W x W images so
+ * many that no SM is idle; nothing is launched.  out[4]:
+ *   out[0]  1: 128-pixel tiles (0, tiles of whole image rows, is not returned
+ *           any more: no kernel takes them)
+ *   out[1]  0 (image rows of such a tile)
+ *   out[2]  output-channel blocks
  *   out[3]  channels per block (the last block may be narrower)
  * Returns ISAM_ERR_UNSUPPORTED for channel counts isam_dwsep_conv rejects.
  */

@@ -581,13 +581,38 @@ int isam_dwsep_plan_info(int W, int Cin, int Cout, int *out) {
     int rc;
     DeviceState *ds = device_state(&rc);
     if (!ds) return rc;
-    return dwsep_plan(W, Cin, Cout, ds->max_smem_optin, out);
+    return dwsep_blocks(W, Cin, Cout, ds->max_smem_optin, out);
 }
 
 int isam_dwsep_plan_for(int W, int Cin, int Cout, int smem_optin, int *out) {
     if (W < 1 || Cin < 1 || Cout < 1 || smem_optin < 1 || !out)
         return set_error(ISAM_ERR_INVALID_ARG, "isam_dwsep_plan_for: sizes must be >= 1, out non-null");
-    return dwsep_plan(W, Cin, Cout, smem_optin, out);
+    return dwsep_blocks(W, Cin, Cout, smem_optin, out);
+}
+
+namespace {
+int dwsep_plan_out(int N, int H, int W, int Cin, int Cout, int num_sms, int smem_optin, int *out) {
+    DwsepPlan p;
+    if (const int rc = dwsep_plan(N, H, W, Cin, Cout, num_sms, smem_optin, &p)) return rc;
+    const int v[9] = {p.patch_w, p.patch_h, p.patches, p.blocks, p.block_cout, p.ctas, p.stages_p, p.stages_a, p.smem};
+    memcpy(out, v, sizeof v);
+    return ISAM_OK;
+}
+}  // namespace
+
+int isam_dwsep_call_info(int N, int H, int W, int Cin, int Cout, int *out) {
+    if (N < 1 || H < 1 || W < 1 || Cin < 1 || Cout < 1 || !out)
+        return set_error(ISAM_ERR_INVALID_ARG, "isam_dwsep_call_info: sizes must be >= 1, out non-null");
+    int rc;
+    DeviceState *ds = device_state(&rc);
+    if (!ds) return rc;
+    return dwsep_plan_out(N, H, W, Cin, Cout, ds->num_sms, ds->max_smem_optin, out);
+}
+
+int isam_dwsep_call_for(int N, int H, int W, int Cin, int Cout, int num_sms, int smem_optin, int *out) {
+    if (N < 1 || H < 1 || W < 1 || Cin < 1 || Cout < 1 || num_sms < 1 || smem_optin < 1 || !out)
+        return set_error(ISAM_ERR_INVALID_ARG, "isam_dwsep_call_for: sizes and limits must be >= 1, out non-null");
+    return dwsep_plan_out(N, H, W, Cin, Cout, num_sms, smem_optin, out);
 }
 
 namespace {

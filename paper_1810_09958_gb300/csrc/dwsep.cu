@@ -45,18 +45,8 @@ struct DwPatchParams {
     uint32_t *err;
 };
 
-// Width of the channel blocks of layers without a row-ring plan: the largest
-// whose weights fit beside two whole A tiles, the staging buffers and the taps.
-// (dwsep_patch_kernel needs less: its A ring holds single 64-channel chunks.)
-__host__ __device__ inline int dw_patch_budget(int Cin, int Cout) {
-    const int atoms = (Cin + 63) / 64;
-    const int nchunks = (Cout + 63) / 64;
-    return 2 * atoms * kBM * 128 + atoms * nchunks * 8192 + 4 * 2 * 4096 + ((9 * Cin * 4) + 1023) / 1024 * 1024 + 256 + 1024;
-}
-
 constexpr int kPatchStagesMax = 4;
 constexpr int kAStagesMax = 4;
-constexpr int kRingMax = 32;     // most rows of a whole-row tiling
 constexpr int kPGroups = 2;
 constexpr int kPProdWarps = kPGroups * kChunkWarps;
 constexpr int kPLoadWarp = kPProdWarps;
@@ -379,96 +369,87 @@ DwPatchKernel dw_patch_kernel_for(int pw) {
 }
 
 // ---------------------------------------------------------------- host side
-// Shared memory of a whole-row tiling: a ring of input rows (each followed by
-// at least one pixel of zeros), one A tile, the block's weights, staging.
-int dw_row_budget(int W, int Cin, int Cout, int ring) {
-    const int atoms = (Cin + 63) / 64;
-    const int nchunks = (Cout + 63) / 64;
-    const int lead = (Cin * 2 + 127) / 128 * 128, row = (W * Cin * 2 + Cin * 2 + 127) / 128 * 128;
-    return (lead + ring * row + 1023) / 1024 * 1024 + atoms * kBM * 128 + atoms * nchunks * 8192 + 4 * 2 * 4096 +
-           8 * (kRingMax + 8) + 16 + 1024;
+bool dw_channels_ok(int Cin, int Cout) {
+    return Cin % 16 == 0 && Cin >= 16 && Cin <= 256 && Cout % 16 == 0 && Cout >= 16 && Cout <= 256;
 }
 
-// Image rows a 128-pixel tile could hold for a block of pc output channels, or 0
-// (an image wider than that, or no ring that fits beside the block's weights).
-int dw_rows_per_tile(int W, int Cin, int pc, int smem_optin) {
-    int rt = W <= kBM ? kBM / W : 0;
-    if (rt > (kRingMax - 2) / 2) rt = (kRingMax - 2) / 2;
-    while (rt > 1 && dw_row_budget(W, Cin, pc, 2 * rt + 2) > smem_optin) --rt;
-    return (rt >= 1 && dw_row_budget(W, Cin, pc, 2 * rt + 2) <= smem_optin) ? rt : 0;
-}
+// Channels of a block when `blocks` share them out (one block has them all).
+int dw_step(int Cout, int blocks) { return blocks == 1 ? Cout : ((Cout + blocks - 1) / blocks + 31) / 32 * 32; }
 
-bool dw_block_fits(int W, int Cin, int pc, int smem_optin) {
-    return dw_rows_per_tile(W, Cin, pc, smem_optin) > 0 || dw_patch_budget(Cin, pc) <= smem_optin;
+// Fewest blocks of the output channels whose weights fit beside two patch chunks and
+// two A chunks; 0 if none does.
+int dw_fewest_blocks(int Cin, int Cout, int pw, int smem_optin) {
+    int blocks = 1;
+    while (dw_patch_layout(Cin, dw_step(Cout, blocks), pw, 2, 2).total > smem_optin) {
+        if (dw_step(Cout, blocks) <= 32) return 0;
+        ++blocks;
+    }
+    const int step = dw_step(Cout, blocks);
+    return (Cout + step - 1) / step;
 }
 
 }  // namespace
 
-// Output channels in blocks of pc (a multiple of 16), planned for the larger of
-// the shared-memory budgets above.  Returns the block width, 0 if none fits.
-int dw_block_width(int W, int Cin, int Cout, int smem_optin) {
-    for (int blocks = 1; blocks <= Cout / 16; ++blocks) {
-        const int pc = ((Cout + blocks - 1) / blocks + 15) / 16 * 16;
-        if (dw_block_fits(W, Cin, pc, smem_optin)) return pc;
+int dwsep_plan(int N, int H, int W, int Cin, int Cout, int num_sms, int smem_optin, DwsepPlan *plan) {
+    if (!dw_channels_ok(Cin, Cout))
+        return set_error(ISAM_ERR_UNSUPPORTED,
+                         "isam_dwsep_conv: needs Cin and Cout multiples of 16 in [16, 256] "
+                         "(Cin=%d Cout=%d)",
+                         Cin, Cout);
+    const long long M = static_cast<long long>(N) * H * W;
+    if (M > (1ll << 31) - 256)
+        return set_error(ISAM_ERR_UNSUPPORTED, "isam_dwsep_conv: N*H*W too large");
+    DwsepPlan p;
+    p.patch_w = dw_patch_width(H, W);
+    p.patch_h = kBM / p.patch_w;
+    p.patches = N * ((H + p.patch_h - 1) / p.patch_h) * ((W + p.patch_w - 1) / p.patch_w);  // at most N * H * W
+    // Blocks share the output channels out: as few as the resident weights allow,
+    // since each recomputes the depthwise stage, but as many as idle SMs can take (a
+    // CTA's start loads its share of the weights, and its tail drains its share of
+    // the last tile: 32 x 14 x 14, 256 -> 256, 64 patches: 17.8 us as two launches, 9.2
+    // as two grid rows).
+    p.blocks = dw_fewest_blocks(Cin, Cout, p.patch_w, smem_optin);
+    if (p.blocks < 1)
+        return set_error(ISAM_ERR_UNSUPPORTED, "isam_dwsep_conv: Cin=%d does not fit shared memory", Cin);
+    while (2LL * p.blocks * p.patches <= num_sms && dw_step(Cout, 2 * p.blocks) >= 64) p.blocks *= 2;
+    p.block_cout = dw_step(Cout, p.blocks);
+    p.blocks = (Cout + p.block_cout - 1) / p.block_cout;
+    p.ctas = std::min(p.patches, std::max(1, num_sms / p.blocks));
+    p.stages_p = kPatchStagesMax;
+    p.stages_a = kAStagesMax;
+    while (dw_patch_layout(Cin, p.block_cout, p.patch_w, p.stages_p, p.stages_a).total > smem_optin) {
+        // The A ring gives way first: a patch takes longer to come.
+        if (p.stages_a > 2)
+            --p.stages_a;
+        else
+            --p.stages_p;
     }
-    return 0;
+    p.smem = dw_patch_layout(Cin, p.block_cout, p.patch_w, p.stages_p, p.stages_a).total;
+    *plan = p;
+    return ISAM_OK;
 }
 
-int dwsep_plan(int W, int Cin, int Cout, int smem_optin, int *out) {
-    if (Cin % 16 != 0 || Cin < 16 || Cin > 256 || Cout % 16 != 0 || Cout < 16 || Cout > 256)
+int dwsep_blocks(int W, int Cin, int Cout, int smem_optin, int *out) {
+    if (!dw_channels_ok(Cin, Cout))
         return set_error(ISAM_ERR_UNSUPPORTED, "isam_dwsep_plan_info: needs Cin and Cout multiples of 16 in [16, 256]");
-    const int pc = dw_block_width(W, Cin, Cout, smem_optin);
-    if (pc < 1) return set_error(ISAM_ERR_UNSUPPORTED, "isam_dwsep_plan_info: Cin=%d does not fit shared memory", Cin);
-    const int rt = dw_rows_per_tile(W, Cin, pc, smem_optin);
-    out[0] = rt > 0 ? 0 : 1;
-    out[1] = rt;
-    out[2] = (Cout + pc - 1) / pc;
-    out[3] = pc;
+    const int blocks = dw_fewest_blocks(Cin, Cout, dw_patch_width(W, W), smem_optin);
+    if (blocks < 1) return set_error(ISAM_ERR_UNSUPPORTED, "isam_dwsep_plan_info: Cin=%d does not fit shared memory", Cin);
+    out[0] = 1;
+    out[1] = 0;
+    out[2] = blocks;
+    out[3] = dw_step(Cout, blocks);
     return ISAM_OK;
 }
 
 int dwsep_launch(int N, int H, int W, int Cin, int Cout, const uint16_t *x, const uint16_t *dw,
                  const uint16_t *pw, float *out, DeviceState &ds, cudaStream_t stream) {
-    if (Cin % 16 != 0 || Cin < 16 || Cin > 256 || Cout % 16 != 0 || Cout < 16 || Cout > 256)
-        return set_error(ISAM_ERR_UNSUPPORTED,
-                         "isam_dwsep_conv: needs Cin and Cout multiples of 16 in [16, 256] "
-                         "(Cin=%d Cout=%d)",
-                         Cin, Cout);
+    DwsepPlan plan;
+    int rc = dwsep_plan(N, H, W, Cin, Cout, ds.num_sms, ds.max_smem_optin, &plan);
+    if (rc) return rc;
     if ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(dw) |
          reinterpret_cast<uintptr_t>(pw) | reinterpret_cast<uintptr_t>(out)) & 15u)
         return set_error(ISAM_ERR_UNSUPPORTED, "isam_dwsep_conv: pointers must be 16-byte aligned");
-    const long long M = static_cast<long long>(N) * H * W;
-    if (M > (1ll << 31) - 256)
-        return set_error(ISAM_ERR_UNSUPPORTED, "isam_dwsep_conv: N*H*W too large");
-    const int px_w = dw_patch_width(H, W), px_h = kBM / px_w;  // patch width and height
-    const int ty = (H + px_h - 1) / px_h, tx = (W + px_w - 1) / px_w;
-    const int tiles = N * ty * tx;  // at most N * H * W
-    // Grid rows share the output channels out: as few as the resident weights
-    // allow, since each recomputes the depthwise stage, but as many as idle SMs
-    // can take (a CTA's start loads its share of the weights, and its tail
-    // drains its share of the last tile: 32 x 14 x 14, 256 -> 256, 64 patches: 17.8
-    // us as two launches, 9.2 as two rows).
-    auto step_for = [&](int rows) { return rows == 1 ? Cout : ((Cout + rows - 1) / rows + 31) / 32 * 32; };
-    auto fits = [&](int rows) {
-        return dw_patch_layout(Cin, step_for(rows), px_w, 2, 2).total <= ds.max_smem_optin;
-    };
-    int rows = 1;
-    while (!fits(rows) && step_for(rows) > 32) ++rows;
-    if (!fits(rows)) return set_error(ISAM_ERR_UNSUPPORTED, "isam_dwsep_conv: Cin=%d does not fit shared memory", Cin);
-    while (2LL * rows * tiles <= ds.num_sms && step_for(2 * rows) >= 64) rows *= 2;
-    const int step = step_for(rows);
-    rows = (Cout + step - 1) / step;
-    int stages_p = kPatchStagesMax, stages_a = kAStagesMax;
-    while (dw_patch_layout(Cin, step, px_w, stages_p, stages_a).total > ds.max_smem_optin) {
-        // The A ring gives way first: a patch takes longer to come.
-        if (stages_a > 2)
-            --stages_a;
-        else
-            --stages_p;
-    }
-    const DwPatchLayout L = dw_patch_layout(Cin, step, px_w, stages_p, stages_a);
     CUtensorMap tmX, tmW, tmOut;
-    int rc;
     auto nhwc = [&](int C, uint64_t elem, uint64_t (&dims)[4], uint64_t (&strides)[3]) {
         const uint64_t px = static_cast<uint64_t>(C) * elem;
         const uint64_t d[4] = {static_cast<uint64_t>(C), static_cast<uint64_t>(W), static_cast<uint64_t>(H),
@@ -479,8 +460,8 @@ int dwsep_launch(int N, int H, int W, int Cin, int Cout, const uint16_t *x, cons
         strides[2] = px * W * H;
     };
     uint64_t dims[4], strides[3];
-    const uint32_t box_x[4] = {64, static_cast<uint32_t>(px_w + 2), static_cast<uint32_t>(px_h + 2), 1};
-    const uint32_t box_o[4] = {32, static_cast<uint32_t>(px_w), static_cast<uint32_t>(32 / px_w), 1};
+    const uint32_t box_x[4] = {64, static_cast<uint32_t>(plan.patch_w + 2), static_cast<uint32_t>(plan.patch_h + 2), 1};
+    const uint32_t box_o[4] = {32, static_cast<uint32_t>(plan.patch_w), static_cast<uint32_t>(32 / plan.patch_w), 1};
     nhwc(Cin, 2, dims, strides);
     if ((rc = make_tmap_4d_bf16(&tmX, x, dims, strides, box_x, false))) return rc;
     nhwc(Cout, 4, dims, strides);
@@ -493,24 +474,23 @@ int dwsep_launch(int N, int H, int W, int Cin, int Cout, const uint16_t *x, cons
     p.W = W;
     p.Cin = Cin;
     p.Cout = Cout;
-    p.step = step;
-    p.ty = ty;
-    p.tx = tx;
-    p.tiles = tiles;
+    p.step = plan.block_cout;
+    p.ty = (H + plan.patch_h - 1) / plan.patch_h;
+    p.tx = (W + plan.patch_w - 1) / plan.patch_w;
+    p.tiles = plan.patches;
     p.atoms = (Cin + 63) / 64;
-    p.nchunks = (step + 63) / 64;
-    p.stages_p = stages_p;
-    p.stages_a = stages_a;
+    p.nchunks = (plan.block_cout + 63) / 64;
+    p.stages_p = plan.stages_p;
+    p.stages_a = plan.stages_a;
     p.dw = dw;
     p.timeout_ns = wait_timeout_ns();
     p.err = ds.err_word;
-    const DwPatchKernel kern = dw_patch_kernel_for(px_w);
+    const DwPatchKernel kern = dw_patch_kernel_for(plan.patch_w);
     if ((rc = ensure_smem_optin(reinterpret_cast<const void *>(kern), ds.max_smem_optin, ds.device,
                                 "cudaFuncSetAttribute(dwsep)")))
         return rc;
-    const int grid = std::min(tiles, std::max(1, ds.num_sms / rows));
-    cudaError_t e = launch_dependent(kern, dim3(static_cast<unsigned>(grid), static_cast<unsigned>(rows)), kPThreads,
-                                     static_cast<size_t>(L.total), stream, 1, tmX, tmW, tmOut, p);
+    cudaError_t e = launch_dependent(kern, dim3(static_cast<unsigned>(plan.ctas), static_cast<unsigned>(plan.blocks)),
+                                     kPThreads, static_cast<size_t>(plan.smem), stream, 1, tmX, tmW, tmOut, p);
     if (e != cudaSuccess) return cuda_error(e, "launch dwsep_patch_kernel");
     return ISAM_OK;
 }

@@ -186,7 +186,18 @@ int dwsep_launch(int N, int H, int W, int Cin, int Cout, const uint16_t *x, cons
 // [3][3][C]; C a multiple of 8, pointers 16-byte aligned (checked by the caller).
 int depthwise_launch(int N, int H, int W, int C, const uint16_t *x, const uint16_t *dw, uint16_t *y,
                      const DeviceState &ds, cudaStream_t s);
-// out[4]: 0 whole image rows per tile or 1 not, image rows per tile, channel blocks, block width.
-int dwsep_plan(int W, int Cin, int Cout, int smem_optin, int *out);
+// How isam_dwsep_conv runs a layer (host arithmetic only).
+struct DwsepPlan {
+    int patch_w = 0, patch_h = 0;  // pixels of a patch, 128 in all
+    int patches = 0;               // of all images
+    int blocks = 0;                // output-channel blocks (grid rows), each with its share of the weights
+    int block_cout = 0;            // channels of one (the last may have fewer)
+    int ctas = 0;                  // CTAs of a block, which walk the patches
+    int stages_p = 0, stages_a = 0;  // 64-channel patch chunks in flight, A chunks
+    int smem = 0;
+};
+int dwsep_plan(int N, int H, int W, int Cin, int Cout, int num_sms, int smem_optin, DwsepPlan *plan);
+// out[4]: 1, 0, fewest channel blocks of W x W images, block width.
+int dwsep_blocks(int W, int Cin, int Cout, int smem_optin, int *out);
 
 }  // namespace isam

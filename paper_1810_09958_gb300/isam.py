@@ -71,6 +71,8 @@ def load():
         lib.isam_depthwise_conv3x3.argtypes = [i, i, i, i, P, P, P]
         lib.isam_dwsep_plan_info.argtypes = [i, i, i, P]
         lib.isam_dwsep_plan_for.argtypes = [i, i, i, i, P]
+        lib.isam_dwsep_call_info.argtypes = [i, i, i, i, i, P]
+        lib.isam_dwsep_call_for.argtypes = [i, i, i, i, i, i, i, P]
         lib.isam_gemm_plan_for.argtypes = [i, i, i, i, i, f, i, i, P, P]
         lib.isam_gemm_chain_for.argtypes = [i, i, i, i, i, f, i, i, P, P]
         lib.isam_gru_plan_info.argtypes = [i, i, i, i, P]
@@ -80,7 +82,8 @@ def load():
                      "isam_gemm_mxfp8", "isam_gemm_grouped_mxfp8",
                      "isam_gru_forward", "isam_gru_forward_reset_before",
                      "isam_gru_forward_stack",
-                     "isam_dwsep_conv", "isam_dwsep_plan_info", "isam_dwsep_plan_for", "isam_depthwise_conv3x3",
+                     "isam_dwsep_conv", "isam_dwsep_plan_info", "isam_dwsep_plan_for", "isam_dwsep_call_info", "isam_dwsep_call_for",
+                     "isam_depthwise_conv3x3",
                      "isam_gru_plan_info", "isam_gru_plan_for", "isam_gemm_plan_for", "isam_gemm_chain_for"):
             getattr(lib, name).restype = ctypes.c_int
         _lib = lib
@@ -367,13 +370,14 @@ def depthwise_conv3x3(N, H, W, C, x, dw_w, y) -> None:
 
 
 _DWSEP_PLAN_KEYS = ("kernel", "rows_per_tile", "blocks", "block_cout")
+_DWSEP_CALL_KEYS = ("patch_w", "patch_h", "patches", "blocks", "block_cout", "ctas", "patch_stages", "a_stages", "smem")
 _GRU_PLAN_KEYS = ("splits", "atoms", "batch_pad", "ctas", "smem", "path", "chunks")
 
 
 def dwsep_plan(W, Cin, Cout, smem_optin=None) -> dict:
-    """isam_dwsep_plan_info: the static tiling of a layer of this width and these
-    channel counts (nothing is launched); with smem_optin, isam_dwsep_plan_for
-    on those limits (no GPU)."""
+    """isam_dwsep_plan_info: the output-channel blocks of a layer of many images of
+    this width and these channel counts (nothing is launched); with smem_optin,
+    isam_dwsep_plan_for on those limits (no GPU)."""
     lib = load()
     out = (ctypes.c_int * 4)()
     if smem_optin is None:
@@ -381,6 +385,18 @@ def dwsep_plan(W, Cin, Cout, smem_optin=None) -> dict:
     else:
         check(lib.isam_dwsep_plan_for(W, Cin, Cout, smem_optin, out))
     return dict(zip(_DWSEP_PLAN_KEYS, list(out)))
+
+
+def dwsep_call(N, H, W, Cin, Cout, num_sms=None, smem_optin=None) -> dict:
+    """isam_dwsep_call_info: how isam_dwsep_conv runs a layer (nothing is launched);
+    with num_sms and smem_optin, isam_dwsep_call_for on those limits (no GPU)."""
+    lib = load()
+    out = (ctypes.c_int * 9)()
+    if num_sms is None:
+        check(lib.isam_dwsep_call_info(N, H, W, Cin, Cout, out))
+    else:
+        check(lib.isam_dwsep_call_for(N, H, W, Cin, Cout, num_sms, smem_optin, out))
+    return dict(zip(_DWSEP_CALL_KEYS, list(out)))
 
 
 def gru_plan(layers, batch, hidden, reset_before=False, num_sms=None, smem_optin=None) -> dict:

@@ -103,36 +103,44 @@ def test_dwsep_ones_window_boundary_pattern():
 
 
 def test_dwsep_benchmark_layer_plan():
-    """The benchmark layer runs as one launch of the row-ring kernel, two
-    image rows (112 pixels) per tile."""
-    assert isam.dwsep_plan(56, 128, 256) == {"kernel": 0, "rows_per_tile": 2, "blocks": 1, "block_cout": 256}
+    """The benchmark layer: 896 patches of 16 x 8 pixels, all output channels in
+    one block, a CTA on every SM."""
+    import torch
+    p = isam.dwsep_call(32, 56, 56, 128, 256)
+    assert (p["patch_w"], p["patch_h"], p["patches"], p["blocks"], p["block_cout"]) == (16, 8, 896, 1, 256)
+    assert p["ctas"] == torch.cuda.get_device_properties(0).multi_processor_count
 
 
-# (N, H, W, Cin, Cout) with the plan the shared-memory budget gives: wide
-# layers whose resident pointwise weights do not fit in one launch run as
-# several output-channel blocks, each block's columns written with the
-# layer's full row pitch (unwritten outputs would keep the canary value).
+# (N, H, W, Cin, Cout) with patch width, channel blocks, channels per block,
+# patch chunks and A chunks in flight: one to four blocks, because the
+# pointwise weights do not fit otherwise or SMs would be idle, each block's
+# columns written with the layer's full row pitch (unwritten outputs would
+# keep the canary value).
 BLOCKED = [
-    ((2, 5, 8, 256, 256), (0, 6, 2, 128)),     # row ring, 6 rows per tile, 2 blocks
-    ((1, 6, 56, 192, 256), (0, 1, 2, 128)),    # row ring, one row per tile, 2 blocks
-    ((1, 4, 56, 256, 256), (1, 0, 4, 64)),     # per-pixel kernel, 4 blocks
-    ((1, 3, 130, 256, 256), (1, 0, 4, 64)),    # wider than one MMA block
-    ((2, 3, 130, 208, 80), (1, 0, 2, 48)),     # 48-wide blocks (a 16-column TMEM tail)
-    ((2, 4, 130, 144, 208), (1, 0, 2, 112)),
-    # the row ring with idle producer threads (52 and 36 channel groups do
-    # not divide the producers; the threads past the last whole segment only
-    # join the barriers)
-    ((2, 3, 11, 208, 80), (0, 5, 1, 80)),
-    ((2, 4, 33, 144, 208), (0, 1, 1, 208)),
-    ((3, 2, 1, 256, 256), (0, 15, 2, 128)),    # one-pixel-wide images
+    ((2, 5, 8, 256, 256), (16, 4, 64, 4, 4)),
+    ((1, 6, 56, 192, 256), (16, 4, 64, 4, 4)),
+    ((1, 4, 56, 256, 256), (32, 4, 64, 4, 3)),
+    ((1, 3, 130, 256, 256), (32, 4, 64, 4, 3)),
+    ((2, 3, 130, 208, 80), (32, 2, 64, 4, 3)),     # a last block of 16 channels (a 16-column TMEM tail)
+    ((2, 4, 130, 144, 208), (32, 4, 64, 4, 4)),
+    ((2, 3, 11, 208, 80), (16, 2, 64, 4, 4)),
+    ((2, 4, 33, 144, 208), (32, 4, 64, 4, 4)),
+    ((3, 2, 1, 256, 256), (16, 4, 64, 4, 4)),      # one-pixel-wide images
+    ((1, 7, 9, 96, 144), (16, 3, 64, 4, 4)),       # three blocks
+    ((9, 41, 70, 192, 208), (8, 1, 208, 2, 2)),    # one block; the weights leave two patch chunks
+    ((200, 3, 40, 80, 208), (32, 1, 208, 3, 2)),
+    ((160, 2, 5, 144, 144), (16, 1, 144, 3, 2)),
+    ((160, 2, 5, 16, 208), (16, 1, 208, 4, 4)),
+    ((160, 2, 30, 208, 208), (32, 2, 128, 3, 2)),  # two blocks although every SM is busy
+    ((160, 2, 5, 256, 240), (16, 2, 128, 4, 2)),
 ]
 
 
 @pytest.mark.parametrize("shape,plan", BLOCKED, ids=[str(s[0]) for s in BLOCKED])
 def test_dwsep_channel_blocks(shape, plan):
     N, H, W, Cin, Cout = shape
-    got_plan = isam.dwsep_plan(W, Cin, Cout)
-    assert (got_plan["kernel"], got_plan["rows_per_tile"], got_plan["blocks"], got_plan["block_cout"]) == plan
+    p = isam.dwsep_call(N, H, W, Cin, Cout)
+    assert (p["patch_w"], p["blocks"], p["block_cout"], p["patch_stages"], p["a_stages"]) == plan
     x, dw, pw = synth.dwsep_operands(N, H, W, Cin, Cout, seed=sum(shape) * 17 + Cout)
     got = run_dwsep(x, dw, pw)
     ref = oracle.dwsep(x, dw, pw)
@@ -140,9 +148,9 @@ def test_dwsep_channel_blocks(shape, plan):
 
 
 def test_dwsep_channel_blocks_integer_bit_exact():
-    """256 -> 256 channels in two blocks of 128: exact on integer data."""
+    """256 -> 256 channels in four blocks of 64: exact on integer data."""
     N, H, W, Cin, Cout = 2, 5, 8, 256, 256
-    assert isam.dwsep_plan(W, Cin, Cout)["blocks"] == 2
+    assert isam.dwsep_call(N, H, W, Cin, Cout)["blocks"] == 4
     x = synth.bf16_integers(11, (N, H, W, Cin), -3, 3)
     dw = synth.bf16_integers(12, (3, 3, Cin), -2, 2)
     pw = synth.bf16_integers(13, (Cin, Cout), -2, 2)
@@ -168,6 +176,8 @@ def test_dwsep_unsupported_rejected():
 def test_dwsep_plan_on_the_device_matches_the_host_plan():
     for (W, cin, cout) in [(56, 128, 256), (56, 256, 256), (8, 256, 256), (130, 48, 16)]:
         assert isam.dwsep_plan(W, cin, cout) == isam.dwsep_plan(W, cin, cout, smem_optin=232448)
+        for (N, H) in [(1, 3), (32, 56)]:
+            assert isam.dwsep_call(N, H, W, cin, cout) == isam.dwsep_call(N, H, W, cin, cout, num_sms=152, smem_optin=232448)
 
 
 # ---- the depthwise factor alone (isam_depthwise_conv3x3) and the unfused

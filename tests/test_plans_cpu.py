@@ -1,5 +1,5 @@
 """The GEMM, GRU and depthwise-separable planners, run on the host through
-the C ABI (isam_gemm_plan_for, isam_gru_plan_for, isam_dwsep_plan_for: host
+the C ABI (isam_gemm_plan_for, isam_gru_plan_for, isam_dwsep_call_for and others: host
 arithmetic, no CUDA call) with a GB300's limits: 152 SMs, 232448 bytes of
 opt-in shared memory per CTA.  Every shape inside the boundary's support
 limits (GRU: batch <= 256, hidden any multiple of 32 up to 1024; dwsep: Cin
@@ -113,20 +113,40 @@ def test_dwsep_every_supported_shape_has_a_plan():
                 pc, blocks = p["block_cout"], p["blocks"]
                 assert pc % 16 == 0 and 16 <= pc <= cout, (W, cin, cout, p)
                 assert blocks == math.ceil(cout / pc) and (blocks - 1) * pc < cout
-                if p["kernel"] == 0:
-                    rt = p["rows_per_tile"]
-                    assert W <= 128 and rt >= 1 and rt * W <= 128, (W, cin, cout, p)
-                else:
-                    assert p["kernel"] == 1 and p["rows_per_tile"] == 0
+                assert p["kernel"] == 1 and p["rows_per_tile"] == 0
+
+
+@pytest.mark.parametrize("N,H,W", [(1, 1, 1), (1, 28, 28), (3, 7, 130), (32, 56, 56), (200, 3, 40), (40, 90, 30)])
+def test_dwsep_calls_fit_the_device(N, H, W):
+    """What isam_dwsep_conv launches, for every pair of channel counts."""
+    for cin in range(16, 257, 16):
+        for cout in range(16, 257, 16):
+            p = isam.dwsep_call(N, H, W, cin, cout, num_sms=SMS, smem_optin=SMEM)
+            pw, ph = p["patch_w"], p["patch_h"]
+            assert pw in (8, 16, 32) and pw * ph == 128
+            assert p["patches"] == N * math.ceil(H / ph) * math.ceil(W / pw)
+            pc, blocks = p["block_cout"], p["blocks"]
+            assert blocks == math.ceil(cout / pc) and (pc == cout or pc % 32 == 0 and pc <= 256), (cin, cout, p)
+            assert 1 <= p["ctas"] <= p["patches"] and p["ctas"] * blocks <= SMS
+            assert 2 <= p["patch_stages"] <= 4 and 2 <= p["a_stages"] <= 4
+            # Weights, A chunks, staging, patches with their halo, taps.
+            atoms, chunks = math.ceil(cin / 64), math.ceil(pc / 64)
+            need = (atoms * chunks * 8192 + p["a_stages"] * 16384 + 8 * 4096 +
+                    p["patch_stages"] * (pw + 2) * (ph + 2) * 128 + 9 * atoms * 128)
+            assert need < p["smem"] <= SMEM, (cin, cout, p)
+            # The blocks of the layer that keeps every SM busy, or more of them.
+            full = isam.dwsep_plan(W, cin, cout, smem_optin=SMEM)["blocks"]
+            assert blocks >= full - 1 and (blocks <= full or p["patches"] * blocks <= SMS)
 
 
 def test_dwsep_benchmark_and_wide_layer_plans():
-    assert isam.dwsep_plan(56, 128, 256, smem_optin=SMEM) == {"kernel": 0, "rows_per_tile": 2, "blocks": 1,
+    assert isam.dwsep_plan(56, 128, 256, smem_optin=SMEM) == {"kernel": 1, "rows_per_tile": 0, "blocks": 1,
                                                               "block_cout": 256}
-    assert isam.dwsep_plan(56, 256, 256, smem_optin=SMEM) == {"kernel": 1, "rows_per_tile": 0, "blocks": 4,
-                                                              "block_cout": 64}
+    assert isam.dwsep_plan(56, 256, 256, smem_optin=SMEM) == {"kernel": 1, "rows_per_tile": 0, "blocks": 2,
+                                                              "block_cout": 128}
     # More shared memory, fewer blocks: the planner follows the limit it is given.
-    assert isam.dwsep_plan(56, 256, 256, smem_optin=400 * 1024)["blocks"] < 4
+    assert isam.dwsep_plan(56, 256, 256, smem_optin=400 * 1024)["blocks"] < 2
+    assert isam.dwsep_call(32, 56, 56, 256, 256, num_sms=SMS, smem_optin=400 * 1024)["blocks"] == 1
 
 
 def test_dwsep_plan_rejects_unsupported_channels():
@@ -139,6 +159,11 @@ def test_dwsep_plan_rejects_unsupported_channels():
     out = (ctypes.c_int * 4)()
     assert lib.isam_dwsep_plan_for(0, 16, 16, SMEM, out) == isam.ISAM_ERR_INVALID_ARG
     assert lib.isam_dwsep_plan_for(8, 16, 16, SMEM, None) == isam.ISAM_ERR_INVALID_ARG
+    out = (ctypes.c_int * 9)()
+    assert lib.isam_dwsep_call_for(1, 8, 8, 24, 16, SMS, SMEM, out) == isam.ISAM_ERR_UNSUPPORTED
+    assert lib.isam_dwsep_call_for(1 << 20, 1 << 10, 8, 16, 16, SMS, SMEM, out) == isam.ISAM_ERR_UNSUPPORTED
+    assert lib.isam_dwsep_call_for(1, 0, 8, 16, 16, SMS, SMEM, out) == isam.ISAM_ERR_INVALID_ARG
+    assert lib.isam_dwsep_call_for(1, 8, 8, 16, 16, SMS, SMEM, None) == isam.ISAM_ERR_INVALID_ARG
 
 
 # ---- the GEMM planner (isam_gemm_plan_for): cluster capacities of 2, 4 and 8
