@@ -185,6 +185,30 @@ int isam_gemm_grouped_fp8(int count, const int *M, const int *N, const int *K, c
                           float *const *C);
 
 /*
+ * How isam_gemm_grouped (e4m3 = 0) or isam_gemm_grouped_fp8 (e4m3 = 1; transA
+ * and transB may be null) runs a group of these sizes; nothing is launched.
+ * out[4]:
+ *   out[0]  CTAs of a cluster that share a tile along K (1, 2, 4 or 8)
+ *   out[1]  1 where the tiles travel with a list, which gives each to the CTA
+ *           that is free first; 0 where CTA i takes tiles i, i + grid, ...
+ *   out[2]  CTAs launched
+ *   out[3]  stages of the operand ring
+ * A group of one is the planned single GEMM.  Errors as for the calls, and
+ * ISAM_ERR_INVALID_ARG for a null out.
+ */
+int isam_gemm_grouped_plan_info(int count, const int *M, const int *N, const int *K, const int *transA,
+                                const int *transB, int e4m3, int *out);
+
+/*
+ * The same for a device with num_sms SMs, smem_optin bytes of shared memory per
+ * CTA and cluster_caps[3] resident clusters of 2, 4 and 8 CTAs; host
+ * arithmetic only, no CUDA call.
+ */
+int isam_gemm_grouped_plan_for(int count, const int *M, const int *N, const int *K, const int *transA,
+                               const int *transB, int e4m3, int num_sms, int smem_optin,
+                               const int *cluster_caps, int *out);
+
+/*
  * The tile plan isam_gemm would use for this problem, chosen by the
  * library's analytic cost model (the paper's "Approach" interface for
  * tiling and device-allocation choices, Sections 3.4 and 4).  Nothing is
@@ -467,6 +491,15 @@ int isam_dwsep_plan_for(int W, int Cin, int Cout, int smem_optin, int *out);
  * ISAM_ERR_INVALID_ARG for sizes < 1, reset_before not 0 or 1, or a null out.
  */
 int isam_gru_plan_info(int layers, int batch, int hidden, int reset_before, int *out);
+
+/*
+ * What of a GRU call runs in one launch on the current device, which is asked
+ * how many clusters it holds; nothing is launched.  out[2]:
+ *   out[0]  layers (2 for pairs in one kernel; fewer at the end of a stack)
+ *   out[1]  batch chunks of a layer
+ * Errors as for isam_gru_plan_info.
+ */
+int isam_gru_launch_info(int layers, int T, int batch, int hidden, int reset_before, int *out);
 
 /*
  * isam_gru_plan_info's plan for a device with num_sms SMs (152 on a GB300)

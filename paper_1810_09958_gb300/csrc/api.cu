@@ -391,6 +391,49 @@ int isam_gemm_grouped_fp8(int count, const int *M, const int *N, const int *K, c
     return gemm_grouped_launch(count, g, *ds, current_stream());
 }
 
+namespace {
+// The route of a group for ds's limits; `who` names the call in errors.
+int grouped_route(const char *who, int count, const int *M, const int *N, const int *K, const int *transA,
+                  const int *transB, int e4m3, const DeviceState *ds, int *out) {
+    if (count < 1 || count > 64) return set_error(ISAM_ERR_INVALID_ARG, "%s: count must be in [1, 64]", who);
+    if (!M || !N || !K || !out || (!e4m3 && (!transA || !transB)) || (e4m3 != 0 && e4m3 != 1))
+        return set_error(ISAM_ERR_INVALID_ARG, "%s: null array, or e4m3 not 0 or 1", who);
+    GemmDesc g[64];
+    int rc;
+    for (int i = 0; i < count; ++i) {
+        g[i] = GemmDesc{M[i], N[i], K[i], e4m3 ? 0 : transA[i], e4m3 ? 1 : transB[i], 1.0f, 0.0f,
+                        reinterpret_cast<const uint16_t *>(16), reinterpret_cast<const uint16_t *>(16),
+                        reinterpret_cast<float *>(16), nullptr, e4m3};
+        if ((rc = gemm_validate(g[i]))) return rc;
+    }
+    if (!ds && !(ds = device_state(&rc))) return rc;
+    GroupedPlan plan;
+    if ((rc = gemm_grouped_plan(count, g, *ds, &plan))) return rc;
+    out[0] = plan.split;
+    out[1] = plan.listed;
+    out[2] = plan.grid;
+    out[3] = plan.stages;
+    return ISAM_OK;
+}
+}  // namespace
+
+int isam_gemm_grouped_plan_info(int count, const int *M, const int *N, const int *K, const int *transA,
+                                const int *transB, int e4m3, int *out) {
+    return grouped_route("isam_gemm_grouped_plan_info", count, M, N, K, transA, transB, e4m3, nullptr, out);
+}
+
+int isam_gemm_grouped_plan_for(int count, const int *M, const int *N, const int *K, const int *transA,
+                               const int *transB, int e4m3, int num_sms, int smem_optin, const int *cluster_caps,
+                               int *out) {
+    if (!cluster_caps || num_sms < 1 || smem_optin < 1 || cluster_caps[0] < 1 || cluster_caps[1] < 1 || cluster_caps[2] < 1)
+        return set_error(ISAM_ERR_INVALID_ARG, "isam_gemm_grouped_plan_for: null capacities or limits < 1");
+    DeviceState ds;  // no device: the limits come from the arguments
+    ds.num_sms = num_sms;
+    ds.max_smem_optin = smem_optin;
+    for (int i = 0; i < 3; ++i) ds.cluster_cap[i] = cluster_caps[i];
+    return grouped_route("isam_gemm_grouped_plan_for", count, M, N, K, transA, transB, e4m3, &ds, out);
+}
+
 int isam_depthwise_conv3x3(int N, int H, int W, int C, const isam_bf16 *x, const isam_bf16 *dw_w, isam_bf16 *y) {
     if (N < 1 || H < 1 || W < 1 || C < 1)
         return set_error(ISAM_ERR_INVALID_ARG, "isam_depthwise_conv3x3: sizes must be >= 1");
@@ -638,6 +681,15 @@ int isam_gru_plan_info(int layers, int batch, int hidden, int reset_before, int 
     DeviceState *ds = device_state(&rc);
     if (!ds) return rc;
     return gru_plan_out(layers, batch, hidden, reset_before, ds->num_sms, ds->max_smem_optin, out);
+}
+
+int isam_gru_launch_info(int layers, int T, int batch, int hidden, int reset_before, int *out) {
+    if (layers < 1 || T < 1 || batch < 1 || hidden < 1 || (reset_before != 0 && reset_before != 1) || !out)
+        return set_error(ISAM_ERR_INVALID_ARG, "isam_gru_launch_info: sizes must be >= 1, reset_before 0 or 1");
+    int rc;
+    DeviceState *ds = device_state(&rc);
+    if (!ds) return rc;
+    return gru_together(layers, T, batch, hidden, reset_before, *ds, &out[0], &out[1]);
 }
 
 int isam_gru_plan_for(int layers, int batch, int hidden, int reset_before, int num_sms, int smem_optin, int *out) {

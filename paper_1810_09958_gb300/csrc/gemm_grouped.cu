@@ -17,6 +17,7 @@
 #include <cstdlib>
 #include <cstdio>
 #include <cstring>
+#include <memory>
 #include <mutex>
 #include <numeric>
 
@@ -585,9 +586,9 @@ float share_out(const GroupParams &p, int workers, const float *cost, uint16_t *
 // The list gives each tile to the CTA that is free first, where that ends at
 // least 3% before the walk.  A group of unlike problems otherwise hands the CTAs
 // that hold the longest K as many further tiles as the others: 18 problems with K
-// from 72 to 6424 62.2 -> 55.5 us, 16 with K from 112 to 5656 34.8 -> 27.4.  The
-// benchmark's sweeps, alike in K, keep the walk, whose CTAs stay on neighbouring
-// panels.
+// from 72 to 6424 62.2 -> 55.5 us, 16 with K from 112 to 5656 34.8 -> 27.4, the
+// benchmark's bf16 sweep (K from 1760 to 4096) 126.8 -> 124.8; its E4M3 form takes
+// 38.6 either way.
 //
 // A split (by 2, 4 or 8, where the device holds that many clusters) shortens the
 // longest tile but costs each one an exchange and a new CTA, so it pays where
@@ -595,10 +596,15 @@ float share_out(const GroupParams &p, int workers, const float *cost, uint16_t *
 // and 32.5 -> 13.1 us, E4M3 group of 3 with K to 7520 21.2 -> 8.6.  (Over 24 drawn
 // groups the geometric mean is 25.2 us without it, 23.0 with 0.5 to 1.5 us for a new
 // CTA, 24.0 with 2.7.)  Above two tiles per SM it is not tried.
+//
+// ISAM_GROUP_ROUTE=walk, list, 2, 4 or 8 (CTAs that split a tile) forces one of them
+// where the group allows it, for tests and measurements.
 void split_rule(GroupParams &p, int grid, const DeviceState &ds) {
     p.listed = 0;
     p.log_split = 0;
     if (p.total_tiles > kMaxListed || grid > kMaxListCtas) return;
+    const char *force = getenv("ISAM_GROUP_ROUTE");
+    if (force && strcmp(force, "walk") == 0) return;
     float cost[kMaxGroup], walk[kMaxListCtas] = {};
     uint16_t owner[kMaxListed];
     bool tall = false;
@@ -612,9 +618,12 @@ void split_rule(GroupParams &p, int grid, const DeviceState &ds) {
     }
     const float walked = *std::max_element(walk, walk + grid);
     float longest = share_out(p, grid, cost, owner);
-    const bool list = longest <= 0.97f * walked;
+    const bool list = force ? strcmp(force, "list") == 0 : longest <= 0.97f * walked;
     if (!list) longest = walked;
-    if (!tall && p.total_tiles <= 2 * grid) {
+    if (force && !tall)
+        for (int ls = 1; ls <= 3; ++ls)
+            if (atoi(force) == 1 << ls && gemm_cluster_capacity(ds, 1 << ls) >= 1) p.log_split = ls;
+    if (!force && !tall && p.total_tiles <= 2 * grid) {
         float best = 0.95f * (longest + 4.2f) - 4.2f;  // 4.2 us: launch, first data, last stores
         for (int ls = 1; ls <= 3; ++ls) {
             const int clusters = std::min(gemm_cluster_capacity(ds, 1 << ls), ds.num_sms >> ls);
@@ -641,20 +650,9 @@ void split_rule(GroupParams &p, int grid, const DeviceState &ds) {
     for (int t = 0; t < p.total_tiles; ++t) p.list[at[owner[t]]++] = static_cast<uint16_t>(t);
 }
 
-}  // namespace
-
-int gemm_grouped_launch(int count, const GemmDesc *g, DeviceState &ds, cudaStream_t stream) {
-    if (count < 1 || count > kMaxGroup)
-        return set_error(ISAM_ERR_INVALID_ARG, "isam_gemm_grouped: count must be in [1, %d]", kMaxGroup);
-    if (count == 1) {
-        // Nothing to share the launch with: the planned tiles and split of a
-        // single call.  Against this kernel, E4M3 / bf16: 384 x 128 x 4096 18.6 / 33.0
-        // -> 5.9 / 7.1 us, 8192 x 256 x 8192 33.7 / 62.2 -> 25.5 / 47.1, 8192 x 8192 x
-        // 1024 144 / 208 -> 75 / 98.
-        GemmPlan plan;
-        if (const int rc = gemm_plan(g[0], ds, &plan)) return rc;
-        return gemm_launch(g[0], plan, ds, stream);
-    }
+// Fills p for a group of two or more but for its tensor maps; order[i]: the caller's
+// index of problem i.  Host arithmetic only.
+void group_plan(int count, const GemmDesc *g, const DeviceState &ds, GroupParams &p, int *order, int *grid_out) {
     auto atoms = [&](int i) { return (g[i].K + (g[i].fp8 ? 2 * kBK : kBK) - 1) / (g[i].fp8 ? 2 * kBK : kBK); };
     // Tile height: 256 rows (two 128-row panels sharing each B block) for
     // problems whose 128-row panel of A is 640 KB or more, which halves the
@@ -681,13 +679,10 @@ int gemm_grouped_launch(int count, const GemmDesc *g, DeviceState &ds, cudaStrea
     }
     // Host-side order: problems with the costliest tiles first, so the
     // round-robin walk over tiles ends with the cheap ones.
-    int order[kMaxGroup];
     std::iota(order, order + count, 0);
     std::stable_sort(order, order + count,
                      [&](int a, int b) { return atoms(a) * panels[a] > atoms(b) * panels[b]; });
 
-    static GroupParams p;  // ~29 KB: built under the lock, copied into the launch
-    std::lock_guard<std::mutex> lk(g_group_mu);
     memset(&p, 0, sizeof p);
     p.count = count;
     int tiles = 0;
@@ -710,6 +705,55 @@ int gemm_grouped_launch(int count, const GemmDesc *g, DeviceState &ds, cudaStrea
         pr.beta = d.beta;
         pr.C = d.C;
         tiles += pr.m_tiles * pr.n_tiles;
+    }
+    p.total_tiles = tiles;
+    int grid = std::min(tiles, ds.num_sms);
+    split_rule(p, grid, ds);
+    if (p.log_split > 0) {
+        grid = tiles << p.log_split;  // one tile per cluster: those that do not fit yet take turns
+        for (int i = 0; i < count; ++i) p.recv_bytes = std::max(p.recv_bytes, partial_bytes(p.prob[i].bn));
+    }
+    int st = 8;
+    while (st > 2 && group_smem_bytes(st, p.recv_bytes) > static_cast<size_t>(ds.max_smem_optin)) --st;
+    p.stages = st;
+    *grid_out = grid;
+}
+
+}  // namespace
+
+int gemm_grouped_plan(int count, const GemmDesc *g, const DeviceState &ds, GroupedPlan *plan) {
+    if (count == 1) {
+        GemmPlan one;
+        if (const int rc = gemm_plan(g[0], ds, &one)) return rc;
+        *plan = GroupedPlan{one.split, 0, one.grid, one.stages};
+        return ISAM_OK;
+    }
+    const auto p = std::make_unique<GroupParams>();
+    int order[kMaxGroup], grid = 0;
+    group_plan(count, g, ds, *p, order, &grid);
+    *plan = GroupedPlan{1 << p->log_split, p->listed, grid, p->stages};
+    return ISAM_OK;
+}
+
+int gemm_grouped_launch(int count, const GemmDesc *g, DeviceState &ds, cudaStream_t stream) {
+    if (count < 1 || count > kMaxGroup)
+        return set_error(ISAM_ERR_INVALID_ARG, "isam_gemm_grouped: count must be in [1, %d]", kMaxGroup);
+    if (count == 1) {
+        // Nothing to share the launch with: the planned tiles and split of a
+        // single call.  Against this kernel, E4M3 / bf16: 384 x 128 x 4096 18.6 / 33.0
+        // -> 5.9 / 7.1 us, 8192 x 256 x 8192 33.7 / 62.2 -> 25.5 / 47.1, 8192 x 8192 x
+        // 1024 144 / 208 -> 75 / 98.
+        GemmPlan plan;
+        if (const int rc = gemm_plan(g[0], ds, &plan)) return rc;
+        return gemm_launch(g[0], plan, ds, stream);
+    }
+    static GroupParams p;  // ~29 KB: built under the lock, copied into the launch
+    std::lock_guard<std::mutex> lk(g_group_mu);
+    int order[kMaxGroup], grid = 0;
+    group_plan(count, g, ds, p, order, &grid);
+    for (int s = 0; s < count; ++s) {
+        const GemmDesc &d = g[order[s]];
+        const GroupProblem &pr = p.prob[s];
         int rc;
         if (pr.fp8) {
             // 128-element (128-byte) K atoms of both K-major E4M3 operands.
@@ -731,19 +775,9 @@ int gemm_grouped_launch(int count, const GemmDesc *g, DeviceState &ds, cudaStrea
             if (rc) return rc;
         }
     }
-    p.total_tiles = tiles;
-    int grid = std::min(tiles, ds.num_sms);
-    split_rule(p, grid, ds);
-    if (p.log_split > 0) {
-        grid = tiles << p.log_split;  // one tile per cluster: those that do not fit yet take turns
-        for (int i = 0; i < count; ++i) p.recv_bytes = std::max(p.recv_bytes, partial_bytes(p.prob[i].bn));
-    }
-    int st = 8;
-    while (st > 2 && group_smem_bytes(st, p.recv_bytes) > static_cast<size_t>(ds.max_smem_optin)) --st;
-    p.stages = st;
     p.timeout_ns = wait_timeout_ns();
     p.err = ds.err_word;
-    const size_t smem = group_smem_bytes(st, p.recv_bytes);
+    const size_t smem = group_smem_bytes(p.stages, p.recv_bytes);
     if (const int rc = ensure_smem_optin(reinterpret_cast<const void *>(gemm_group_kernel), ds.max_smem_optin,
                                          ds.device, "cudaFuncSetAttribute(grouped gemm)"))
         return rc;

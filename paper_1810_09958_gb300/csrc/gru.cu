@@ -808,6 +808,27 @@ int gru_empty_rings(uint16_t *hx, size_t bytes, cudaStream_t stream) {
     return e == cudaSuccess ? ISAM_OK : cuda_error(e, "emptying the GRU exchange rings");
 }
 
+// Chunks (or layers) of hidden H, gru_cta_count(H) CTAs each in clusters of its K
+// splits, that kern keeps resident at once with `smem` bytes a CTA.
+cudaError_t gru_resident(GruKernel kern, int H, size_t smem, int *chunks) {
+    const int ks = gru_splits(H);
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = static_cast<unsigned>(ks);
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3(static_cast<unsigned>(gru_cta_count(H)), 1, 1);
+    cfg.blockDim = dim3(kThreads, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int clusters = 0;
+    const cudaError_t e = cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg);
+    *chunks = clusters * ks / gru_cta_count(H);
+    return e;
+}
+
 // Fills the shape fields of p and launches the
 // recurrence: one cluster of KS CTAs per group of 32 units, as a plain cluster
 // launch after checking that every cluster fits on the device at once (the
@@ -844,15 +865,15 @@ int launch_recurrent(GruParams &p, const CUtensorMap &tmWn, size_t smem, cudaStr
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     const GruKernel kern = layers > 1 ? gru_poll_kernel_for(p.ks) : gru_kernel_for(p.ks, bp);
-    int max_clusters = 0;
-    cudaError_t e = cudaOccupancyMaxActiveClusters(&max_clusters, kern, &cfg);
+    int resident = 0;
+    cudaError_t e = gru_resident(kern, H, smem, &resident);
     if (e != cudaSuccess) return cuda_error(e, "cudaOccupancyMaxActiveClusters(gru)");
     // Chunks on the device at once; all layers have to be.
-    const int fit = std::min(rings, max_clusters * p.ks / p.n_cta);
+    const int fit = std::min(rings, resident);
     if (fit < layers || fit < 1)
         return set_error(ISAM_ERR_UNSUPPORTED,
-                         "GRU recurrence: %d CTAs in clusters of %d cannot be co-resident (%d clusters fit)",
-                         p.n_cta, p.ks, max_clusters);
+                         "GRU recurrence: %d x %d CTAs in clusters of %d cannot be co-resident (%d x %d fit)",
+                         layers, p.n_cta, p.ks, resident, p.n_cta);
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.numAttrs = gru_dependent(p.T * (p.reset_before ? 2 : 1)) ? 2 : 1;
@@ -966,27 +987,35 @@ int gru_plan(int layers, int batch, int hidden, int reset_before, int num_sms, i
 // 1 GB of projections between them.
 static int gru_layers_together(int layers, int H, size_t gx_floats, const DeviceState &ds) {
     const int ks = gru_splits(H);
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = static_cast<unsigned>(ks);
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.gridDim = dim3(static_cast<unsigned>(gru_cta_count(H)), 1, 1);
-    cfg.blockDim = dim3(kThreads, 1, 1);
-    cfg.dynamicSmemBytes = gru_smem_bytes(H, true);
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    int clusters = 0;
+    int resident = 0;
     if (ensure_smem_optin(reinterpret_cast<const void *>(gru_poll_kernel_for(ks)), ds.max_smem_optin, ds.device,
                           "cudaFuncSetAttribute(gru)") != ISAM_OK ||
-        cudaOccupancyMaxActiveClusters(&clusters, gru_poll_kernel_for(ks), &cfg) != cudaSuccess) {
+        gru_resident(gru_poll_kernel_for(ks), H, gru_smem_bytes(H, true), &resident) != cudaSuccess) {
         (void)cudaGetLastError();
         return 1;
     }
     const size_t set_bytes = static_cast<size_t>(ks) * gx_floats * sizeof(float);
     const long long by_size = 1 + static_cast<long long>((static_cast<size_t>(1) << 30) / set_bytes);
-    return static_cast<int>(std::max<long long>(1, std::min<long long>({layers, clusters * ks / gru_cta_count(H), by_size})));
+    return static_cast<int>(std::max<long long>(1, std::min<long long>({layers, resident, by_size})));
+}
+
+int gru_together(int layers, int T, int batch, int hidden, int reset_before, const DeviceState &ds, int *layers_together,
+                 int *chunks_together) {
+    GruPlan plan;
+    int rc = gru_plan(layers, batch, hidden, reset_before, ds.num_sms, ds.max_smem_optin, &plan);
+    if (rc) return rc;
+    const size_t gx_floats = static_cast<size_t>(T) * batch * 3 * hidden;
+    *layers_together = plan.path == 1 ? 2 : plan.path == 2 ? gru_layers_together(layers, hidden, gx_floats, ds) : 1;
+    *chunks_together = 1;
+    if (plan.chunks > 1) {
+        if ((rc = gru_smem_attr(ds.max_smem_optin, ds.device))) return rc;
+        int resident = 0;
+        const cudaError_t e = gru_resident(gru_kernel_for(plan.ks, plan.bp), hidden, gru_smem_bytes(hidden, false, plan.bp),
+                                           &resident);
+        if (e != cudaSuccess) return cuda_error(e, "cudaOccupancyMaxActiveClusters(gru)");
+        *chunks_together = std::max(1, std::min(plan.chunks, resident));
+    }
+    return ISAM_OK;
 }
 
 int gru_stack_launch(int layers, int T, int batch, int hidden, int reset_before, const uint16_t *x,

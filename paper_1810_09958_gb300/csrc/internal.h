@@ -130,6 +130,13 @@ int gemm_pair_launch(const GemmDesc &g, const GemmPlan &plan, DeviceState &ds, c
 
 // Independent GEMMs in one persistent launch (1 <= count <= 64).
 int gemm_grouped_launch(int count, const GemmDesc *g, DeviceState &ds, cudaStream_t s);
+// How that launch runs its tiles (host arithmetic only, given the cluster capacities).
+struct GroupedPlan {
+    int split;   // CTAs of a cluster that share a tile along K (1: none do)
+    int listed;  // 1: the tiles travel with a list, 0: the CTAs walk them
+    int grid, stages;
+};
+int gemm_grouped_plan(int count, const GemmDesc *g, const DeviceState &ds, GroupedPlan *plan);
 
 // Block-scaled E4M3 GEMM (OCP MX): C = alpha (SA o A)(SB o B)^T + beta C with
 // A M x K and B N x K E4M3 bytes (K-major) and one E8M0 scale byte per 32 K
@@ -172,6 +179,9 @@ struct GruPlan {
     int chunks = 0;   // batch chunks per layer
 };
 int gru_plan(int layers, int batch, int hidden, int reset_before, int num_sms, int smem_optin, GruPlan *g);
+// Layers and batch chunks of a call that share a launch on the current device.
+int gru_together(int layers, int T, int batch, int hidden, int reset_before, const DeviceState &ds, int *layers_together,
+                 int *chunks_together);
 int gru_wave_launch(int T, int batch, int H, const float *gx_a, const uint16_t *U_a, const uint16_t *W_b,
                     const uint16_t *U_b, const float *b_a, const float *b_b, const float *h0_a,
                     const float *h0_b, float *out_a, float *out_b, uint16_t *hx, DeviceState &ds,

@@ -76,6 +76,9 @@ def load():
         lib.isam_gemm_plan_for.argtypes = [i, i, i, i, i, f, i, i, P, P]
         lib.isam_gemm_chain_for.argtypes = [i, i, i, i, i, f, i, i, P, P]
         lib.isam_gru_plan_info.argtypes = [i, i, i, i, P]
+        lib.isam_gru_launch_info.argtypes = [i, i, i, i, i, P]
+        lib.isam_gemm_grouped_plan_info.argtypes = [i, P, P, P, P, P, i, P]
+        lib.isam_gemm_grouped_plan_for.argtypes = [i, P, P, P, P, P, i, i, i, P, P]
         lib.isam_gru_plan_for.argtypes = [i, i, i, i, i, i, P]
         for name in ("isam_version", "isam_set_stream", "isam_sync", "isam_shutdown", "isam_gemm",
                      "isam_gemm_plan_info", "isam_gemm_plan_info2", "isam_gemm_grouped", "isam_gemm_fp8", "isam_gemm_grouped_fp8",
@@ -84,7 +87,8 @@ def load():
                      "isam_gru_forward_stack",
                      "isam_dwsep_conv", "isam_dwsep_plan_info", "isam_dwsep_plan_for", "isam_dwsep_call_info", "isam_dwsep_call_for",
                      "isam_depthwise_conv3x3",
-                     "isam_gru_plan_info", "isam_gru_plan_for", "isam_gemm_plan_for", "isam_gemm_chain_for"):
+                     "isam_gru_plan_info", "isam_gru_plan_for", "isam_gru_launch_info", "isam_gemm_plan_for",
+                     "isam_gemm_chain_for", "isam_gemm_grouped_plan_info", "isam_gemm_grouped_plan_for"):
             getattr(lib, name).restype = ctypes.c_int
         _lib = lib
         return lib
@@ -287,6 +291,23 @@ def gemm_grouped(problems) -> None:
     GroupedGemm(problems)()
 
 
+def grouped_plan(sizes, e4m3=False, num_sms=None, smem_optin=None, cluster_caps=None) -> dict:
+    """isam_gemm_grouped_plan_info: how a group of (M, N, K, transA, transB), or (M, N, K)
+    with e4m3, runs its tiles (nothing is launched); with num_sms, smem_optin and
+    cluster_caps, isam_gemm_grouped_plan_for on those limits (no GPU)."""
+    lib = load()
+    n = len(sizes)
+    cols = [(ctypes.c_int * n)(*[int(v) for v in col]) for col in zip(*sizes)]
+    cols += [None] * (5 - len(cols))
+    out = (ctypes.c_int * 4)()
+    if num_sms is None:
+        check(lib.isam_gemm_grouped_plan_info(n, *cols, int(e4m3), out))
+    else:
+        caps = (ctypes.c_int * 3)(*cluster_caps)
+        check(lib.isam_gemm_grouped_plan_for(n, *cols, int(e4m3), num_sms, smem_optin, caps, out))
+    return dict(zip(("split", "listed", "grid", "stages"), list(out)))
+
+
 def gemm_plan(M, N, K, transA, transB, beta=0.0, num_sms=None, smem_optin=None, cluster_caps=None) -> dict:
     """The tile plan the library's cost model picks (nothing is launched);
     with num_sms, smem_optin and cluster_caps (resident clusters of 2, 4, 8
@@ -410,3 +431,11 @@ def gru_plan(layers, batch, hidden, reset_before=False, num_sms=None, smem_optin
     else:
         check(lib.isam_gru_plan_for(layers, batch, hidden, int(bool(reset_before)), num_sms, smem_optin, out))
     return dict(zip(_GRU_PLAN_KEYS, list(out)))
+
+
+def gru_launch(layers, T, batch, hidden, reset_before=False) -> dict:
+    """isam_gru_launch_info: layers and batch chunks that share a launch on the
+    current device (nothing is launched)."""
+    out = (ctypes.c_int * 2)()
+    check(load().isam_gru_launch_info(layers, T, batch, hidden, int(bool(reset_before)), out))
+    return {"layers": out[0], "chunks": out[1]}

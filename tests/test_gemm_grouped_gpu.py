@@ -63,22 +63,45 @@ def test_grouped_unlike_problems_odd_widths(beta):
     widths = [1, 3, 9, 31, 33, 77, 126, 129, 255, 40]
     ks = [3000, 8, 520, 72, 1000, 64, 264, 2040, 136, 16]
     specs = [(1500 + 131 * i, N, K, 0, 1, 2.0, beta) for i, (N, K) in enumerate(zip(widths, ks))]
-    assert sum(-(-M // 128) * -(-N // 128) for M, N, *_ in specs) > 152
+    plan = isam.grouped_plan([s[:5] for s in specs])
+    assert plan["listed"] == 1 and plan["split"] == 1
     for (got, ref), spec in zip(run_group(specs, dist="int4", seed0=700), specs):
         assert np.array_equal(got.astype(np.float64), ref), spec
 
 
-@pytest.mark.parametrize("specs", [
-    # few tiles, so that clusters of 8 split them along K: also where K has fewer
-    # atoms than the cluster CTAs (9 and 72)
-    [(300, 40, 4096), (200, 77, 72), (130, 9, 2048), (64, 200, 16)],
-    # more tiles than clusters of 8 or 4 fit
-    [(4000, 16, 4096), (2500, 100, 2048), (700, 33, 520)],
-], ids=["few", "more"])
+# Few tiles, which clusters of 8 split along K, also where K has fewer atoms than
+# the cluster has CTAs (16 and 72); more tiles, which clusters of 2 split.
+FEW = [(300, 40, 4096), (200, 77, 72), (130, 9, 2048), (64, 200, 16)]
+MORE = [(4000, 16, 4096), (2500, 100, 2048), (700, 33, 520)]
+
+
+@pytest.mark.parametrize("specs,split", [(FEW, 8), (MORE, 2)], ids=["few", "more"])
 @pytest.mark.parametrize("beta", [0.0, -1.0])
-def test_grouped_tiles_split_along_k(specs, beta):
+def test_grouped_tiles_split_along_k(specs, split, beta):
     specs = [(M, N, K, 0, 1, 2.0, beta) for M, N, K in specs]
+    assert isam.grouped_plan([s[:5] for s in specs])["split"] == split
     for (got, ref), spec in zip(run_group(specs, dist="int4", seed0=800), specs):
+        assert np.array_equal(got.astype(np.float64), ref), spec
+
+
+# Sizes for every way to run a group's tiles, E4M3 too (K a multiple of 16): 34 tiles,
+# more than clusters of 8 fit at once.
+ROUTES = [(300, 40, 1040), (200, 77, 80), (2600, 9, 528), (64, 200, 16), (257, 129, 1008)]
+
+
+@pytest.mark.parametrize("route", ["walk", "list", "2", "4", "8"])
+@pytest.mark.parametrize("e4m3", [False, True], ids=["bf16", "e4m3"])
+def test_grouped_routes_give_the_same_sums(route, e4m3, monkeypatch):
+    monkeypatch.setenv("ISAM_GROUP_ROUTE", route)
+    plan = isam.grouped_plan(ROUTES if e4m3 else [s + (0, 1) for s in ROUTES], e4m3)
+    assert plan["listed"] == (route == "list") and plan["split"] == (int(route) if route.isdigit() else 1)
+    if e4m3:
+        specs = [(M, N, K, 2.0, -1.0) for M, N, K in ROUTES]
+        res = run_group_fp8(specs, dist="int", seed0=1700)
+    else:
+        specs = [(M, N, K, 0, 1, 2.0, -1.0) for M, N, K in ROUTES]
+        res = run_group(specs, dist="int4", seed0=1700)
+    for (got, ref), spec in zip(res, specs):
         assert np.array_equal(got.astype(np.float64), ref), spec
 
 

@@ -62,12 +62,14 @@ def test_gru_stack_two_layers_benchmark_shape(reset_before):
         assert nmax_err(got[l], ref[l]) <= TOL, (l, nmax_err(got[l], ref[l]))
 
 
-@pytest.mark.parametrize("L,T,batch,H,rb", [
+@pytest.mark.parametrize("L,T,batch,H,rb,together", [
     # layers that share a launch: 1, 2 and 4 K splits, one step, many steps, more
-    # layers than fit together (5 at 38 CTAs each, 3 at 104)
-    (3, 1, 32, 32, False), (5, 40, 7, 160, False), (4, 33, 32, 480, True), (3, 64, 20, 576, False),
-    (5, 6, 32, 608, False), (3, 5, 11, 832, False), (2, 50, 1, 96, True)])
-def test_gru_stack_layers_share_a_launch(L, T, batch, H, rb):
+    # layers than fit together (5 at 38 CTAs each, 3 at 52, 2 at 120)
+    (3, 1, 32, 32, False, 3), (5, 40, 7, 160, False, 5), (4, 33, 32, 480, True, 4), (3, 64, 20, 576, False, 3),
+    (5, 6, 32, 608, False, 4), (3, 5, 11, 832, False, 2), (2, 50, 1, 96, True, 2), (3, 9, 5, 256, True, 3),
+    (2, 4, 6, 960, False, 1)])
+def test_gru_stack_layers_share_a_launch(L, T, batch, H, rb, together):
+    assert isam.gru_launch(L, T, batch, H, rb)["layers"] == together
     x, W, U, b, h0 = synth.gru_stack_operands(L, T, batch, H, seed=L * 31 + T * 7 + batch + H)
     got = run_stack(x, W, U, b, h0, rb)
     ref = oracle.gru_stack(x, W, U, b, h0, reset_before=rb)

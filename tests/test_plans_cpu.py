@@ -276,3 +276,49 @@ def test_gemm_argument_rules_on_the_host():
     for (M, N, K, tA, tB), want in cases:
         got = lib.isam_gemm_plan_for(M, N, K, tA, tB, 0.0, SMS, SMEM, caps, out)
         assert got == want, ((M, N, K, tA, tB), got, isam.last_error())
+
+
+# ---- the route of a group's tiles (isam_gemm_grouped_plan_for)
+def grouped(sizes, e4m3=False):
+    return isam.grouped_plan(sizes, e4m3, num_sms=SMS, smem_optin=SMEM, cluster_caps=[76, 36, 16])
+
+
+def test_grouped_routes(monkeypatch):
+    monkeypatch.delenv("ISAM_GROUP_ROUTE", raising=False)
+    alike = [(8192, 128, 1024)] * 8                     # 512 tiles of one kind: walked
+    unlike = [(1500 + 131 * i, 33, 72 * (1 + i * i)) for i in range(12)]  # K from 72 to 8784: listed
+    few = [(300, 40, 4096), (200, 77, 72)]              # 5 tiles: split
+    assert grouped([s + (0, 1) for s in alike]) == {"split": 1, "listed": 0, "grid": SMS, "stages": 7}
+    assert grouped([s + (0, 1) for s in unlike])["listed"] == 1
+    p = grouped([s + (0, 1) for s in few])
+    assert p["split"] == 8 and p["grid"] == 5 * 8 and p["listed"] == 0
+    # A group of one is the planned single GEMM.
+    one, g = grouped([(512, 96, 512, 1, 0)]), gemm_plan(512, 96, 512, 1, 0, caps=[76, 36, 16])
+    assert (one["split"], one["grid"], one["stages"]) == (g["split"], g["grid"], g["stages"])
+    # More tiles than a list holds: walked whatever the sizes.
+    assert grouped([(8192, 2048, 64 * (1 + i), 0, 1) for i in range(4)])["listed"] == 0
+    # E4M3 groups by the same rule.
+    assert grouped([(300, 40, 4096), (200, 77, 80)], e4m3=True)["split"] == 8
+
+
+@pytest.mark.parametrize("route", ["walk", "list", "2", "4", "8"])
+def test_grouped_route_can_be_forced(route, monkeypatch):
+    monkeypatch.setenv("ISAM_GROUP_ROUTE", route)
+    p = grouped([(300, 40, 1040, 0, 1), (2600, 9, 528, 0, 1)])
+    assert p["listed"] == (route == "list") and p["split"] == (int(route) if route.isdigit() else 1)
+
+
+def test_grouped_plan_rejects_bad_arguments():
+    import ctypes
+    lib = isam.load()
+    out, caps, v = (ctypes.c_int * 4)(), (ctypes.c_int * 3)(76, 36, 16), (ctypes.c_int * 2)(64, 64)
+    z = (ctypes.c_int * 2)(0, 0)
+    f = lib.isam_gemm_grouped_plan_for
+    assert f(0, v, v, v, z, z, 0, SMS, SMEM, caps, out) == isam.ISAM_ERR_INVALID_ARG
+    assert f(2, v, v, v, None, z, 0, SMS, SMEM, caps, out) == isam.ISAM_ERR_INVALID_ARG
+    assert f(2, v, v, v, z, z, 2, SMS, SMEM, caps, out) == isam.ISAM_ERR_INVALID_ARG
+    assert f(2, v, v, v, z, z, 0, SMS, SMEM, None, out) == isam.ISAM_ERR_INVALID_ARG
+    assert f(2, v, v, v, z, z, 0, SMS, SMEM, caps, None) == isam.ISAM_ERR_INVALID_ARG
+    k = (ctypes.c_int * 2)(64, 12)
+    assert f(2, v, v, k, z, z, 0, SMS, SMEM, caps, out) == isam.ISAM_ERR_UNSUPPORTED
+    assert f(2, v, v, v, None, None, 1, SMS, SMEM, caps, out) == isam.ISAM_OK
