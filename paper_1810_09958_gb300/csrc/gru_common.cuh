@@ -160,14 +160,17 @@ __device__ __forceinline__ void push_rows(uint32_t acc, int half, int npiece, ui
     tc_fence_before();
 }
 
-// How partial rows cross the cluster: as bulk copies of whole rows, or as
+// How partial rows cross the cluster: as bulk copies of whole half rows, or as
 // 16-byte stores of the pieces that hold the batch.  The stores of a warp go to
-// 32 different rows and take longer than the copies once a row is about five
-// eighths full: 64 steps at hidden 1024 (stores / copies) take 162 / 179 us at
-// batch 8, 174 / 176 at 20, 179 / 177 at 24, 198 / 185 at 32, 312 / 286 at 64;
-// at 128 padded rows the two are equal at a full batch (527 / 529) and the
-// stores ahead below it (441 / 482 at 96).
-__host__ __device__ inline bool gru_push_bulk(int batch, int bp) { return bp < 128 && 8 * batch > 5 * bp; }
+// 32 different rows and take longer than the copies once a row is about three
+// quarters full, at every hidden size: 40 steps (stores / copies) take 111.6 / 115.4
+// us at hidden 1024 and batch 20, 115.7 / 116.0 at 24, 121.2 / 114.9 at 32, 170.6 /
+// 172.1 at 48, 184.5 / 174.9 at 64; hidden 384, two splits: 101.8 / 102.4, 105.2 / 103.4,
+// 112.8 / 107.5, 154.5 / 153.3, 179.1 / 168.0; hidden 256: 85.3 / 89.7, 89.5 / 90.3,
+// 95.1 / 90.1, 133.8 / 136.4, 146.9 / 138.0.  At 128 padded rows (64 steps, hidden
+// 1024) the two are equal at a full batch (527 / 529) and the stores ahead below it
+// (441 / 482 at 96).
+__host__ __device__ inline bool gru_push_bulk(int batch, int bp) { return bp < 128 && 4 * batch >= 3 * bp; }
 
 // Whether a recurrence of this many rounds is a dependent launch, whose set-up
 // overlaps the projection: it starts about 2 us earlier (5 steps, hidden 64: 34.6 ->
