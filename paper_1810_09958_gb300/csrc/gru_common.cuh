@@ -172,12 +172,6 @@ __device__ __forceinline__ void push_rows(uint32_t acc, int half, int npiece, ui
 // (441 / 482 at 96).
 __host__ __device__ inline bool gru_push_bulk(int batch, int bp) { return bp < 128 && 4 * batch >= 3 * bp; }
 
-// Whether a recurrence of this many rounds is a dependent launch, whose set-up
-// overlaps the projection: it starts about 2 us earlier (5 steps, hidden 64: 34.6 ->
-// 33.2 us), but its clusters are placed around the projection's last CTAs and a
-// round takes 0.05 us longer (128 steps of two layers, hidden 1024: 395 -> 402 us).
-inline bool gru_dependent(int rounds) { return rounds <= 24; }
-
 // Staging buffers of push_rows_bulk, which rounds take in turn.
 constexpr int kGruStages = 2;
 

@@ -490,10 +490,14 @@ int gru_wave_launch(int T, int batch, int H, const float *gx_a, const uint16_t *
     if (max_clusters * kKS < p.n_cta)
         return set_error(ISAM_ERR_UNSUPPORTED, "two-layer GRU kernel: %d CTAs in clusters of 4 cannot be co-resident",
                          p.n_cta);
-    // The caller has emptied the rings ahead of the projection.
+    // The caller has emptied the rings ahead of the projection.  A dependent launch
+    // starts about 1.5 us earlier, but its clusters are placed around the projection's
+    // last CTAs and a step takes 0.07 us longer: off / on 34.0 / 32.5 us for 4 steps at
+    // hidden 1024, batch 32, 88.0 / 87.6 for 24, 112.0 / 112.1 for 32, 132.6 / 133.5 for
+    // 40, 378 / 386 for 128.
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.numAttrs = gru_dependent(T) ? 2 : 1;
+    cfg.numAttrs = T <= 32 ? 2 : 1;
     e = cudaLaunchKernelEx(&cfg, gru_wave_kernel, p);
     if (e != cudaSuccess) return cuda_error(e, "launch gru_wave_kernel");
     return ISAM_OK;
