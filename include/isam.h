@@ -12,10 +12,17 @@
  *     allocated and owned by the caller.  The library never frees or keeps
  *     them past the call's completion on the stream.
  *   - Tensors are packed row-major (no leading-dimension arguments).
- *   - The library owns small internal workspaces (an error word per device,
- *     the GRU's input-projection buffer and its hidden-state exchange
- *     buffer).  They are allocated on first use, reused, and released
- *     by isam_shutdown().
+ *   - The library owns internal workspaces, per device: an error word; 2 MB of
+ *     GRU exchange rings; the GRU's input projection, 12 x T x batch x hidden
+ *     bytes; for stacks a bf16 copy of a layer's states (2 x T x batch x hidden
+ *     bytes) or, in the per-layer chain (see isam_gru_plan_info), the layers'
+ *     projections, 12 x T x batch x hidden x splits bytes each: two, or one more
+ *     than the layers that share a launch, as long as those between them stay
+ *     within 1 GB (layers run one after another where no memory is found).  They
+ *     are allocated on first use, grown where a larger call comes, reused, and
+ *     released by isam_shutdown().  A call that allocates cannot be captured into
+ *     a CUDA graph, and a captured graph is good until a call outgrows what it
+ *     uses: the rings never move, the projections not for more layers.
  *
  * Execution
  *   - Every compute call is asynchronous on the stream set by

@@ -308,6 +308,7 @@ int isam_shutdown(void) {
         cudaFree(ds->gru_gx);
         cudaFree(ds->gru_hx);
         cudaFree(ds->gru_gxp);
+        for (int i = 0; i < ds->gru_gxp_olds; ++i) cudaFree(ds->gru_gxp_old[i]);
         cudaFree(ds->gru_xb);
         delete ds;
         g_dev[d] = nullptr;

@@ -788,6 +788,30 @@ int ensure_ws(void **ptr, size_t *cap, size_t need, const char *what) {
     return ISAM_OK;
 }
 
+// Replaces a projection workspace that serves the call as it is by one of `need`
+// bytes, or of twice its own, without freeing it: only layers that could share a
+// launch ask for more, and a graph captured before may still use it.  What is kept
+// adds up to less than the new one.  False (nothing changed) during a capture, which
+// admits no allocation, and where no memory is found.
+bool grow_projections(DeviceState &ds, size_t need, cudaStream_t stream) {
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (ds.gru_gxp_olds == static_cast<int>(sizeof ds.gru_gxp_old / sizeof ds.gru_gxp_old[0]) ||
+        cudaStreamIsCapturing(stream, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    need = std::max(need, 2 * ds.gru_gxp_bytes);
+    float *grown = nullptr;
+    if (cudaMalloc(&grown, need) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    ds.gru_gxp_old[ds.gru_gxp_olds++] = ds.gru_gxp;
+    ds.gru_gxp = grown;
+    ds.gru_gxp_bytes = need;
+    return true;
+}
+
 // Tensor map of the layers' W as [layer, 3 gates][H rows][H] (box: 96 rows of
 // one group over one 64-wide K atom).
 int weight_map(const uint16_t *Wt, int layers, int H, CUtensorMap *tm) {
@@ -800,7 +824,10 @@ int weight_map(const uint16_t *Wt, int layers, int H, CUtensorMap *tm) {
 // Elements of one slot of the exchange ring: [H/8 pieces][bp rows][8].
 int slot_elems(int H, int bp) { return H * bp; }
 
-// Bytes of the whole ring.
+// Bytes of the rings of any call on a GB300.
+constexpr size_t kRingsBytes = static_cast<size_t>(2) << 20;
+
+// Bytes of a whole ring.
 size_t ring_bytes(int H, int bp) { return static_cast<size_t>(kSlots) * slot_elems(H, bp) * sizeof(uint16_t); }
 
 int gru_empty_rings(uint16_t *hx, size_t bytes, cudaStream_t stream) {
@@ -1049,7 +1076,13 @@ int gru_stack_launch(int layers, int T, int batch, int hidden, int reset_before,
     const int ks = gru_splits(H);
     int together = plan.path == 2 ? gru_layers_together(layers, H, gx_floats, ds) : 1;
     const size_t set_floats = static_cast<size_t>(ks) * gx_floats;
-    if (layers > 1 && !chunked) {
+    const size_t sets_held = ds.gru_gxp_bytes / (set_floats * sizeof(float));
+    if (layers > 1 && !chunked && sets_held >= 2) {
+        // Room for one layer after another; more only for layers that can share a launch.
+        if (sets_held < static_cast<size_t>(together) + 1 &&
+            !grow_projections(ds, static_cast<size_t>(together + 1) * set_floats * sizeof(float), stream))
+            together = static_cast<int>(sets_held) - 1;
+    } else if (layers > 1 && !chunked) {
         auto sets = [&] {
             return ensure_ws(reinterpret_cast<void **>(&ds.gru_gxp), &ds.gru_gxp_bytes,
                              static_cast<size_t>(together + 1) * set_floats * sizeof(float),
@@ -1063,11 +1096,13 @@ int gru_stack_launch(int layers, int T, int batch, int hidden, int reset_before,
         }
         if (rc) return rc;
     }
-    // Room for two exchange rings (a layer pair uses both) or one for each chunk
-    // of the batch, whatever the path, so that the buffer moves only when that
-    // grows; each launch empties what it uses.
+    // Exchange rings: two for a layer pair, else one for each chunk of the batch or
+    // layer of a launch, which empties what it uses.  All shapes fit the 2 MB taken
+    // at first (four chunks of 64 rows, or two of 128, at hidden 1024; layers together
+    // hold no more units than the device has SMs for), so the buffer does not move.
     const int rings = std::max(plan.chunks, together);
-    if ((rc = ensure_ws(reinterpret_cast<void **>(&ds.gru_hx), &ds.gru_hx_bytes, std::max(2, rings) * ring_bytes(H, bp),
+    if ((rc = ensure_ws(reinterpret_cast<void **>(&ds.gru_hx), &ds.gru_hx_bytes,
+                        std::max(kRingsBytes, std::max(2, rings) * ring_bytes(H, bp)),
                         "allocating the GRU exchange buffer")))
         return rc;
     if ((rc = gru_smem_attr(ds.max_smem_optin, ds.device))) return rc;

@@ -24,13 +24,17 @@ struct DeviceState {
     // host-side plan for given limits fills them in).
     int cluster_cap[3] = {0, 0, 0};
     uint32_t *err_word = nullptr;  // 4 x uint32 on the device
-    // GRU workspaces (grown on demand).
+    // GRU workspaces (grown on demand; the exchange rings at their largest at once).
     float *gru_gx = nullptr;       // [T*batch][3H] fp32 input projection
     size_t gru_gx_bytes = 0;
-    uint16_t *gru_hx = nullptr;    // bf16 hidden-state exchange ring (two for a layer pair)
+    uint16_t *gru_hx = nullptr;    // bf16 hidden-state exchange rings, one per batch chunk or layer of a launch
     size_t gru_hx_bytes = 0;
-    float *gru_gxp = nullptr;      // 2 x [ks][T*batch][3H] fp32 stacked layers' projections
+    float *gru_gxp = nullptr;      // sets of [ks][T*batch][3H] fp32 stacked layers' projections (two at least)
     size_t gru_gxp_bytes = 0;
+    // Its predecessors that were large enough for a call but not for all the layers
+    // one launch can take: a graph captured before may still use them.
+    float *gru_gxp_old[16] = {};
+    int gru_gxp_olds = 0;
     uint16_t *gru_xb = nullptr;    // [T*batch][H] bf16 states of a layer (next pair's input)
     size_t gru_xb_bytes = 0;
 };

@@ -225,3 +225,71 @@ def test_gru_stack_pair_nan_stays_in_its_sequence():
     got = run_stack(x, W, U, b, h0)
     assert np.isnan(got[:, :, 0]).all()
     assert np.array_equal(got[:, :, 1:], clean[:, :, 1:])
+
+
+# ---- workspaces and CUDA graphs: a call that one workspace serves can be captured,
+# and its graph replayed, whatever the number of layers or chunks of other calls.
+
+def device_stack(L, T, batch, H, seed):
+    import torch
+    x, W, U, b, h0 = synth.gru_stack_operands(L, T, batch, H, seed=seed)
+    out = torch.empty(L * T * batch * H, device="cuda")
+    args = (L, T, batch, H, dev_bf16(x), dev_bf16(W), dev_bf16(U), f32dev(b), None)
+    return (lambda: isam.gru_forward_stack(*args, out)), out
+
+
+def captured(call):
+    import torch
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        call()
+    return graph
+
+
+def test_gru_stack_can_be_captured_after_fewer_layers():
+    T, batch, H = 8, 4, 96
+    isam.sync()
+    isam.shutdown()  # workspaces anew
+    two, out2 = device_stack(2, T, batch, H, 301)
+    five, out5 = device_stack(5, T, batch, H, 302)
+    two()
+    isam.sync()
+    ref2 = out2.clone()
+    graph2, graph5 = captured(two), captured(five)  # five layers in the room of two
+    graph5.replay()
+    isam.sync()
+    ref5 = out5.clone()
+    out5.zero_()
+    assert isam.gru_launch(5, T, batch, H)["layers"] == 5
+    five()  # outside a capture it takes more
+    isam.sync()
+    assert torch_equal(out5, ref5)
+    for graph, out, ref in ((graph2, out2, ref2), (graph5, out5, ref5)):
+        out.zero_()
+        graph.replay()
+        isam.sync()
+        assert torch_equal(out, ref)
+
+
+def test_gru_wider_batch_can_be_captured_after_a_longer_run():
+    import torch
+    H = 64
+    isam.sync()
+    isam.shutdown()
+    long_run, _ = device_stack(1, 16, 64, H, 303)
+    wide, out = device_stack(1, 3, 256, H, 304)
+    long_run()
+    isam.sync()
+    graph = captured(wide)  # four chunks of 64 rows after one
+    graph.replay()
+    isam.sync()
+    ref = out.clone()
+    out.zero_()
+    wide()
+    isam.sync()
+    assert torch_equal(out, ref) and torch.isfinite(ref).all()
+
+
+def torch_equal(a, b):
+    import torch
+    return torch.equal(a, b)
