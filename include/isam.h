@@ -277,7 +277,7 @@ int isam_gemm_chain_for(int M, int N, int K, int transA, int transB, float beta,
  *
  * The input projection for all T steps runs as one GEMM into a library
  * workspace; the recurrence runs in one persistent kernel that keeps U
- * resident in shared memory and multiplies bf16(h_{t-1}) on the tensor cores
+ * resident in tensor memory and multiplies bf16(h_{t-1}) on the tensor cores
  * (h itself is carried in fp32).  Gates are evaluated in fp32.
  *
  * Supported: T >= 1, 1 <= batch <= 256, hidden a multiple of 32 in
@@ -330,26 +330,26 @@ int isam_gru_forward_reset_before(int T, int batch, int hidden, const isam_bf16 
  *   h_out  [layers][T][batch][hidden]    fp32, every layer's states; layer
  *                                        layers - 1 is the stack's output
  *
- With the reset gate after the product and hidden a multiple of 256, layers
+ * With the reset gate after the product and hidden a multiple of 256, layers
  * run in pairs in one persistent kernel: in round r it advances the lower
  * layer to step r and the upper one to step r - 1, computing the upper
  * layer's input projection from the same bf16 tile of the lower layer's
  * states (T + 1 rounds for two layers); between pairs, and for an odd last
  * layer, the states below are rounded to bf16 and projected by the GEMM.
- * Otherwise (the reset-before form, other hidden sizes) layer l's kernel
- * keeps its K quarter of layer l + 1's W resident and multiplies it by the
- * bf16(h_{t-1}) tile it loads for its own recurrent product, so layer
+ * Otherwise (the reset-before form, other hidden sizes) layer l's CTAs
+ * keep their K range of layer l + 1's W resident and multiply it by the
+ * bf16(h_{t-1}) tile they load for their own recurrent product, so layer
  * l + 1's projection is computed while layer l runs (one extra round covers
  * h_{T-1}); layer l + 1 reads it as per-K-rank partial sums (fixed order:
- * deterministic).  Either way the next layer sees bf16(h^l_t), as the
- * recurrent product sees bf16(h_{t-1}).
+ * deterministic), a step or two behind where both fit on the device
+ * together.  Either way the next layer sees bf16(h^l_t), as the recurrent
+ * product sees bf16(h_{t-1}).
  *
  * Supported: as isam_gru_forward (batch up to 256, every multiple of 32
  * for hidden; the K splits are chosen so that both weight slices of the
  * per-layer chain fit).  Batches above 32 run layer by layer: the states
  * below are rounded to bf16 and projected by the GEMM, and each layer's
- * recurrence runs in chunks of padded rows.  Workspace: 2 x ks x T x batch x
- * 3*hidden fp32 (ks = 4, 2 or 1 K splits) beside isam_gru_forward's.
+ * recurrence runs in chunks of padded rows.
  */
 int isam_gru_forward_stack(int layers, int T, int batch, int hidden, int reset_before,
                            const isam_bf16 *x, const isam_bf16 *W, const isam_bf16 *U,

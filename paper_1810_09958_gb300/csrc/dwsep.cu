@@ -91,7 +91,7 @@ __host__ __device__ inline DwPatchLayout dw_patch_layout(int Cin, int Cout, int 
 //   warps 18-25  epilogue, two per TMEM lane quarter.
 //
 // What bounds it: with many patches the output writes (32 x 56 x 56, 128 -> 256
-// at 25.2 us is 5.1 TB/s of unique bytes, a plain copy 6.8), with few the first
+// at 24.3 us is 5.3 TB/s of unique bytes, a plain copy 6.8), with few the first
 // patch's latency (5.6 us for any layer of up to one patch per SM).  Two kernels
 // preceded it.  Whole image rows as tiles, the input rows in a shared-memory
 // ring (widths to 128): its producers walked along the rows with a window of 12
@@ -99,8 +99,8 @@ __host__ __device__ inline DwPatchLayout dw_patch_layout(int Cin, int Cout, int 
 // the layer above; 16 x 112 x 112, 32 -> 64: 29.3 -> 17.1 us; 4 x 14 x 14,
 // 32 -> 48: 9.6 -> 5.6 us.  Nine 16-byte taps an output from L1/L2 (other widths):
 // 5 x 75 x 150, 48 -> 80: 26.0 -> 10.9 us; 2 x 130 x 180, 128 -> 128: 58 -> 13.6 us.
-// Patches in flight on the first layer: 2 / 3 / 4 give 29.6 / 25.8 / 25.1 us; a
-// third A chunk at 3 patches 26.2 us.
+// Patches in flight on the first layer: 2 / 3 / 4 gave 29.6 / 25.8 / 25.1 us and a
+// third A chunk at 3 patches 26.2, before TMA and MMA were issued under elect.sync.
 template <int PW>
 __global__ void __launch_bounds__(kPThreads, 1)
     dwsep_patch_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmW,

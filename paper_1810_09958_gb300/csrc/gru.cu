@@ -140,9 +140,10 @@ __host__ __device__ inline GruLayout gru_layout(int ks, int ka, bool has_next, i
 // MMA's swizzled shared-memory layout.  A published word is then visible one
 // store plus one load later; a release, a counter, its poll and a TMA load
 // (the exchange this replaced) were four such latencies one after another.
-// Hidden 1024, batch 32: 4.77 -> 2.55 us a step (610 -> 343 us for 128 steps);
-// hidden 480, batch 5: 5.0 -> 2.6 us a step.  Of the 2.55 us about 0.8 is the
-// exchange, 0.3 the products, 0.5 push and reduction, 0.3 the gates.
+// Hidden 1024, batch 32: 609 -> 332 us for 128 steps, 2.5 us for one more; hidden
+// 480, batch 5: 100 -> 51 us for 20 steps, 2.0 for one more.  Of the 2.5 us about
+// 0.8 is the exchange, 0.3 the products, 0.5 push and reduction, 0.3 the gates; the
+// rest has not been attributed.
 //
 // The ring is [piece of 8 units][batch row]: a CTA's words fill whole lines that
 // no other CTA writes.  With the rows of 64 units interleaved (8 CTAs writing
@@ -969,9 +970,12 @@ int gru_plan(int layers, int batch, int hidden, int reset_before, int num_sms, i
         auto fits = [&](int cand) {
             return gru_bp_ok(q.ks, cand) && gru_smem_bytes(H, false, cand) <= static_cast<size_t>(smem_optin);
         };
-        // Steps of a wider chunk take longer (4.5 us at 64 padded rows, 8.3 at
-        // 128, hidden 1024), but chunks that do not fit on the device together
-        // run one after another.
+        // Steps of a wider chunk take longer (in proportion 4.5 at 64 padded rows, 8.3
+        // at 128), but chunks that do not fit on the device together run one after
+        // another.  24 steps, hidden / batch in chunks of 64 and of 128: 256 / 128 87 and
+        // 143 us, 512 / 128 98 and 160, 512 / 192 186 and 161, 768 / 96 184 and 149, 1024 /
+        // 128 210 and 188, 1024 / 256 417 and 376; the choice is 1% behind at 192 rows of
+        // hidden 768 and 1024 (292 and 289, 315 and 310).
         const int together = std::max(1, num_sms / q.n_cta);
         double best = 0.0;
         for (const auto &[cand, step_us] : {std::pair<int, double>{64, 4.5}, {128, 8.3}}) {
